@@ -147,8 +147,36 @@ struct swr_plan_s {
     // instead of a final march (tune.superpose < 0, or too little free memory: final march)
     bool superpose = false;
     double2* d_urec = nullptr;
-    std::vector<long long> rec_base;   // per subdomain: Phi_l (nt x n_j), Phi_r, U_d (n_j)
+    std::vector<long long> rec_base;   // per subdomain: Phi_l (nt x rec_n), Phi_r, U_d (n_j)
+    std::vector<int> rec_n;            // entries of one recorded state of subdomain j
     long long* d_rec_base = nullptr;
+    // Fixed-point marches (swr_march_fx.cu) of a list of constant-matrix marches: the build list
+    // (R = 3 right-hand sides per subdomain: zero flux, left, right impulse), its impulses alone
+    // (R = 2: the preconditioner's operator), its zero-flux marches alone (the adjoint's d), and
+    // the marches with flux inputs (R g, the final march).  Subdomains are grouped by the warps a
+    // system takes; one launch per group.
+    struct FxList {
+        const MarchSys* sys = nullptr;   // the list it stands for (NULL: no such list)
+        int nsys = 0, R = 0;
+        bool driven = false;             // flux inputs
+        FxShape sh{};
+        MarchSys* d_sys1 = nullptr;      // the same systems for step 1: state into d_fxu
+        int* d_grp = nullptr;            // [N][R] system indices, in launch order
+        long long* d_soff = nullptr;     // [nsys] offset of a system's state in d_fxu
+        int *d_scale = nullptr, *d_bad = nullptr;   // [nsys] scale of a system, marched in FP64
+        int* d_shift = nullptr;          // [nsys][2][nt] its scalings-down, step by step
+        double2* d_fin = nullptr;        // driven: [nsys][2][nt] converted inputs
+        int* d_tiny = nullptr;           // driven: [nsys] no input
+        struct Launch {
+            int start, count, T;
+        };
+        std::vector<Launch> launches;
+    };
+    FxList fx_build, fx_imp, fx_d, fx_R, fx_final;
+    bool fx_stale[5] = {};               // fsL[] whose fixed-point form is older than its factors
+    bool fac_stale[5] = {};              // fsL[] of another chunk length than the last build's
+    int3* d_subsys = nullptr;            // per subdomain: its systems in the build list
+    double2 *d_fxu = nullptr, *d_fxtrace = nullptr;
     unsigned long long* d_pit = nullptr;   // nonlinear marches: nodes x inner iterations
     double* d_scal = nullptr;      // [0] jump
     Workspace ws;
@@ -356,6 +384,9 @@ struct SegArgs {
     double2* vrec = nullptr;
     const double2* vfwd = nullptr;
     double *gint = nullptr, *gl = nullptr, *gr = nullptr;
+    double2* urec = nullptr;        // recorded states (NULL: the plan's)
+    const int* only = nullptr;      // march only the flagged systems
+    int tstride = 0;                // entries per trace (0: the launch's own step count)
 };
 
 // fixL > 0: the modelled shape for that chunk length (no tuned entry)
@@ -532,7 +563,9 @@ int launch_cfg(swr_plan_t p, const MarchCfg& cfg, int kind, bool zero_potential,
     a.gout = gout;
     a.uT = uT;
     a.trace = trace;
-    a.urec = (!zero_potential && p->superpose) ? p->d_urec : nullptr;
+    a.urec = seg.urec ? seg.urec : ((!zero_potential && p->superpose) ? p->d_urec : nullptr);
+    a.only = seg.only;
+    a.tstride = seg.tstride;
     a.two_sigma = p->two_sigma;
     a.inv_ik = p->inv_ik;
     a.status = p->d_status;
@@ -592,11 +625,70 @@ inline int march_kind(swr_plan_t p, bool zero_potential) {
     return MK_STATIC;
 }
 
+// The fixed-point form of a list's marches: step 1 in FP64 (it sets each system's scale), steps
+// 2..nt in fixed point, the fluxes from the end traces, and the flagged systems again in FP64.
+swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxList& fl,
+                        const double2* gin, double2* gout, double2* uT, double2* trace,
+                        const double2* u0, long long work) {
+    const int L = fl.sh.L;
+    FactorSet& fs = zero_potential ? p->fs0L[lidx(L)] : p->fsL[lidx(L)];
+    if (fs.L != L) return SWR_ERR_STATE;
+    const MarchCfg cfg = march_config(p, fl.nsys, MK_STATIC, L);
+    const int pi = prof_begin(p, 0, work);
+    int rc = 0;
+    if (!zero_potential && p->fx_stale[lidx(L)]) {   // formed by the first march that needs it
+        rc = swr_launch_fx_prepare(fs, p->N, p->s);
+        p->fx_stale[lidx(L)] = rc != 0;
+    }
+    SegArgs first, again;
+    first.urec = p->d_fxu;
+    first.tstride = p->nt;
+    if (!rc)
+        rc = launch_cfg(p, cfg, MK_STATIC, zero_potential, fl.d_sys1, fl.nsys, gin, gout, nullptr,
+                        trace, u0, 1, first);
+    FxMarchArgs a{};
+    a.nt = p->nt;
+    a.C = fl.sh.C;
+    a.R = fl.R;
+    a.sys = fl.sys;
+    a.sub_tc = p->d_tc;
+    a.sub_n = p->d_n;
+    a.sub_goff = p->d_goff;
+    a.soff = fl.d_soff;
+    a.u1 = p->d_fxu;
+    a.urec = (!zero_potential && p->superpose) ? p->d_urec : nullptr;
+    a.uT = uT;
+    a.trace = p->d_fxtrace;
+    a.scale = fl.d_scale;
+    a.bad = fl.d_bad;
+    a.tshift = fl.d_shift;
+    a.status = p->d_status;
+    a.fin = fl.d_fin;
+    a.tiny = fl.d_tiny;
+    a.driven = fl.driven && gin;
+    if (!rc) rc = swr_launch_fx_start(fs, a, fl.nsys, gin, p->inv_ik, p->s);
+    for (const auto& g : fl.launches) {
+        a.grp = fl.d_grp + (size_t)g.start * fl.R;
+        a.T = g.T;
+        if (!rc) rc = swr_launch_march_fx(fs, a, g.count, p->s);
+    }
+    if (!rc) rc = swr_launch_fx_flux(a, fl.nsys, p->two_sigma, gin, gout, trace, p->s);
+    again.only = fl.d_bad;
+    if (!rc)
+        rc = launch_cfg(p, cfg, MK_STATIC, zero_potential, fl.sys, fl.nsys, gin, gout, uT, trace,
+                        u0, p->nt, again);
+    prof_end(p, pi);
+    return rc ? launch_fail("march (fixed point)", __LINE__) : SWR_OK;
+}
+
 // vrec (nonlinear marches only): also record v_n of every step, rows of nx values
 swr_status run_march(swr_plan_t p, bool zero_potential, const MarchSys* d_sys, int nsys,
                      const double2* gin, double2* gout, double2* uT, double2* trace,
                      const double2* u0, long long work, double2* vrec = nullptr) {
     const int kind = march_kind(p, zero_potential);
+    for (const auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final})
+        if (kind == MK_STATIC && fl->sys && fl->sys == d_sys && fl->nsys == nsys && !vrec)
+            return run_march_fx(p, zero_potential, *fl, gin, gout, uT, trace, u0, work);
     const MarchCfg cfg = march_config(p, nsys, kind);
     const int pi = prof_begin(p, kind == MK_NL ? 3 : 0, work);
     SegArgs sa;
@@ -821,7 +913,7 @@ std::vector<MarchSys> build_systems(const swr_plan_s* p, bool with_d) {
     // superposed u(T): every impulse march records its states, the d march its final state
     const bool rec = p->superpose;
     auto slot = [&](int sub, int which, int nt) -> long long {   // 0: Phi_l, 1: Phi_r, 2: U_d
-        return rec ? p->rec_base[sub] + (long long)which * nt * p->n[sub] : 0;
+        return rec ? p->rec_base[sub] + (long long)which * nt * p->rec_n[sub] : 0;
     };
     if (with_d) {   // d = R 0: one march per subdomain, all instances first
         for (const InstInfo& I : p->inst)
@@ -881,6 +973,71 @@ swr_status upload_systems(MarchSys** dst, const std::vector<MarchSys>& v,
     if (st) return st;
     CK(cudaMemcpy(*dst, v.data(), sizeof(MarchSys) * v.size(), cudaMemcpyHostToDevice));
     if (p) p->host_sys.push_back({*dst, v});
+    return SWR_OK;
+}
+
+// Set up the fixed-point form of the systems sys[0..nsys) (host copies hs): R kinds per
+// subdomain, at most one system of each (0 zero flux or driven, 1 left, 2 right impulse; R = 2:
+// the impulses).
+swr_status fx_list(swr_plan_t p, swr_plan_s::FxList& fl, const MarchSys* sys, const MarchSys* hs,
+                   int nsys, int R, const FxShape& sh, bool driven = false) {
+    fl.nsys = nsys;
+    fl.R = R;
+    fl.sh = sh;
+    fl.driven = driven;
+    std::vector<MarchSys> one(hs, hs + nsys);
+    std::vector<long long> soff(nsys);
+    std::vector<int> of((size_t)p->N * R, -1), order(p->N), need(p->N);
+    long long tot = 0;
+    for (int q = 0; q < nsys; ++q) {
+        const int kind = (hs[q].flags & SYS_IMP_L) ? 1 : ((hs[q].flags & SYS_IMP_R) ? 2 : 0);
+        of[(size_t)hs[q].sub * R + kind - (R == 2 ? 1 : 0)] = q;
+        soff[q] = tot;
+        one[q].flags = (hs[q].flags & (SYS_ZERO_U0 | SYS_IMP_L | SYS_IMP_R | SYS_TRACE)) | SYS_REC_LAST;
+        one[q].rec = tot;
+        tot += p->n[hs[q].sub];
+    }
+    // one launch per number of warps a system takes (C = 1), the longest marches first
+    for (int j = 0; j < p->N; ++j) {
+        order[j] = j;
+        need[j] = sh.C > 1 ? sh.T : (chunks_for(p->n[j], sh.L) + 1 + 31) / 32 * 32;
+    }
+    std::vector<int> nts(p->N);
+    for (const InstInfo& I : p->inst)
+        for (int j = 0; j < I.N; ++j) nts[I.sub0 + j] = I.nt;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        return need[a] != need[b] ? need[a] > need[b] : nts[a] > nts[b];
+    });
+    std::vector<int> grp;
+    for (int j : order) {
+        bool any = false;
+        for (int k = 0; k < R; ++k) any |= of[(size_t)j * R + k] >= 0;
+        if (!any) continue;
+        if (fl.launches.empty() || fl.launches.back().T != need[j])
+            fl.launches.push_back({(int)(grp.size() / R), 0, need[j]});
+        fl.launches.back().count += 1;
+        for (int k = 0; k < R; ++k) grp.push_back(of[(size_t)j * R + k]);
+    }
+    swr_status st = upload_systems(&fl.d_sys1, one, p);
+    if (!st) st = dalloc(&fl.d_grp, grp.size());
+    if (!st) st = dalloc(&fl.d_soff, soff.size());
+    if (!st) st = dalloc(&fl.d_scale, (size_t)nsys);
+    if (!st) st = dalloc(&fl.d_bad, (size_t)nsys);
+    if (!st) st = dalloc(&fl.d_shift, (size_t)nsys * 2 * p->nt);
+    if (!st && driven) st = dalloc(&fl.d_fin, (size_t)nsys * 2 * p->nt);
+    if (!st && driven) st = dalloc(&fl.d_tiny, (size_t)nsys);
+    if (!st && !p->d_fxu) {   // shared by the lists: the longest one is set up first
+        st = dalloc(&p->d_fxu, (size_t)tot);
+        if (!st) st = dalloc(&p->d_fxtrace, (size_t)nsys * 2 * p->nt);
+    }
+    if (st) return st;
+    CK(cudaMemcpy(fl.d_grp, grp.data(), sizeof(int) * grp.size(), cudaMemcpyHostToDevice));
+    CK(cudaMemcpy(fl.d_soff, soff.data(), sizeof(long long) * nsys, cudaMemcpyHostToDevice));
+    if (R == 3) {
+        if ((st = dalloc(&p->d_subsys, (size_t)p->N))) return st;
+        CK(cudaMemcpy(p->d_subsys, of.data(), sizeof(int3) * p->N, cudaMemcpyHostToDevice));
+    }
+    fl.sys = sys;
     return SWR_OK;
 }
 
@@ -1498,6 +1655,17 @@ void swr_destroy(swr_plan_t p) {
     cudaFree(p->d_sys_build); cudaFree(p->d_sys_R); cudaFree(p->d_sys_final);
     cudaFree(p->d_status); cudaFree(p->d_scal); cudaFree(p->d_pit);
     cudaFree(p->d_urec); cudaFree(p->d_rec_base);
+    for (auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final}) {
+        cudaFree(fl->d_sys1);
+        cudaFree(fl->d_grp);
+        cudaFree(fl->d_soff);
+        cudaFree(fl->d_scale);
+        cudaFree(fl->d_bad);
+        cudaFree(fl->d_shift);
+        cudaFree(fl->d_fin);
+        cudaFree(fl->d_tiny);
+    }
+    cudaFree(p->d_subsys); cudaFree(p->d_fxu); cudaFree(p->d_fxtrace);
     cudaFree(p->d_W); cudaFree(p->d_spec); cudaFree(p->d_spec0); cudaFree(p->d_Gw);
     cudaFree(p->d_Pwin); cudaFree(p->d_hspec); cudaFree(p->d_hspec0);
     cudaFree(p->d_xspec);
@@ -1744,6 +1912,33 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
             }
         }
     }
+    // Fixed-point marches: constant matrix, Robin or Neumann ends, subdomains within a cluster,
+    // the two-level separator solve allowed, and more than a handful of steps (step 1 runs in
+    // FP64 by itself)
+    const bool force_long = p->tune.long_march >= 1;   // the grid-wide march for any V(x) plan
+    const bool is_long =
+        force_long || chunks_for(p->nmax, 16) + 1 > 16 * march_tmax(MK_STATIC, 16);
+    FxShape fxs{};
+    const bool pot = d->precond == SWR_PC_ZERO_POTENTIAL || d->precond == SWR_PC_MEAN_POTENTIAL;
+    const int fxR = d->vkind == SWR_V_STATIC ? 3 : (pot ? 2 : 0);
+    // a subdomain that waves cross late or not at all keeps too few bits of its cross response
+    // and would be marched twice: reach T / sqrt(dt) at the wavenumber 1 / sqrt(dt), with half
+    // of it to spare
+    bool crossed = true;
+    for (const InstInfo& I : p->inst)
+        for (int j = 0; j < I.N; ++j)
+            crossed = crossed && (p->n[I.sub0 + j] - 1) * p->h <= I.nt * std::sqrt(d->dt);
+    const bool fx = fxR > 0 && d->tc == SWR_TC_ROBIN && !is_long && p->two_level && crossed &&
+                    p->nt >= 16 &&
+                    swr_fx_shape(p->nmax, p->N, fxR, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fxs);
+    // the marches of one system per subdomain (R g, final, the adjoint's d)
+    FxShape fx1{};
+    const bool fx_one = d->vkind == SWR_V_STATIC && d->tc == SWR_TC_ROBIN && !is_long &&
+                        p->two_level && p->nt >= 16 &&
+                        swr_fx_shape(p->nmax, p->N, 1, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fx1);
+    p->rec_n.resize(p->N);
+    for (int j = 0; j < p->N; ++j)   // chunk-element order: (L + 1) rows of P_j + 1
+        p->rec_n[j] = fx && fxR == 3 ? (fxs.L + 1) * (chunks_for(p->n[j], fxs.L) + 1) : p->n[j];
     if (!st && d->vkind == SWR_V_STATIC &&
         (d->tc == SWR_TC_ROBIN ? (d->tc_re != 0.0 || d->tc_im != 0.0) : p->nt < 4260)) {
         // u(T) by superposition: Phi_l, Phi_r (nt x n_j each) and U_d per subdomain, if
@@ -1754,7 +1949,7 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
         for (const InstInfo& I : p->inst)
             for (int j = 0; j < I.N; ++j) {
                 base[I.sub0 + j] = tot;
-                tot += (2LL * I.nt + 1) * p->n[I.sub0 + j];
+                tot += 2LL * I.nt * p->rec_n[I.sub0 + j] + p->n[I.sub0 + j];
             }
         size_t fr = 0, all = 0;
         if (on && cudaMemGetInfo(&fr, &all) == cudaSuccess &&
@@ -1783,9 +1978,18 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
         for (const InstInfo& I : p->inst)
             for (int j = 0; j < I.N; ++j) p->work_R += (long long)p->n[I.sub0 + j] * I.nt;
         st = upload_systems(&p->d_sys_build, vb, p);
+        if (!st && fx && fxR == 3)
+            st = fx_list(p, p->fx_build, p->d_sys_build, vb.data(), p->nsys_build, 3, fxs);
+        if (!st && fx && pot) {
+            FxShape sh = fxs;
+            if (fxR == 2 || swr_fx_shape(p->nmax, p->N, 2, p->forceL == 2 ? 0 : p->forceL, p->nsm, &sh))
+                st = fx_list(p, p->fx_imp, p->d_sys_build + p->N, vb.data() + p->N,
+                             p->nsys_build - p->N, 2, sh);
+        }
+        if (!st && fx_one)
+            st = fx_list(p, p->fx_d, p->d_sys_build, vb.data(), p->N, 1, fx1);
     }
-    const bool force_long = p->tune.long_march >= 1;   // the grid-wide march for any V(x) plan
-    if (!st && (force_long || chunks_for(p->nmax, 16) + 1 > 16 * march_tmax(MK_STATIC, 16))) {
+    if (!st && is_long) {
         // a subdomain longer than one cluster can hold (16 CTAs x 256 chunks of 16 nodes):
         // the grid-wide march, V(x) and single instances only
         if (d->vkind != SWR_V_STATIC || p->batched) {
@@ -1856,6 +2060,12 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
     }
     if (!st) st = upload_systems(&p->d_sys_R, apply_systems(p, 0), p);
     if (!st) st = upload_systems(&p->d_sys_final, apply_systems(p, SYS_WRITE_UT | SYS_TRACE), p);
+    if (!st && fx_one) {
+        auto vr = apply_systems(p, 0), vf = apply_systems(p, SYS_WRITE_UT | SYS_TRACE);
+        st = fx_list(p, p->fx_R, p->d_sys_R, vr.data(), p->N, 1, fx1, true);
+        if (!st && !p->superpose)
+            st = fx_list(p, p->fx_final, p->d_sys_final, vf.data(), p->N, 1, fx1, true);
+    }
     if (!st) {
         for (auto& e : p->ev)
             if (cudaEventCreate(&e) != cudaSuccess) st = SWR_ERR_CUDA;
@@ -1922,8 +2132,11 @@ static swr_status build_body(swr_plan_t p, bool do_assemble) {
         if ((st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od))) return st;
     } else {
         // factorisations for the chunk lengths the marches of this plan will use
-        const int Lb = march_config(p, p->nsys_build).L, La = march_config(p, p->N).L;
+        const bool fx = p->fx_build.sys != nullptr;
+        const int Lb = fx ? p->fx_build.sh.L : march_config(p, p->nsys_build).L;
+        const int La = p->fx_R.sys ? p->fx_R.sh.L : march_config(p, p->N).L;
         if ((st = factor_for(p, p->fsL[lidx(Lb)], Lb, p->d_V, p->d_dg, p->d_od))) return st;
+        if (fx) LK(swr_launch_fx_prepare(p->fsL[lidx(Lb)], p->N, s));
         if (La != Lb && (st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od)))
             return st;
         CK(cudaMemsetAsync(p->d_iface, 0, sizeof(double2) * (nb + (size_t)p->ncols), s));
@@ -1949,8 +2162,10 @@ static swr_status build_body(swr_plan_t p, bool do_assemble) {
             Vp = p->d_Vbar;
         }
         if ((st = assemble(p, Vp, p->d_dg0, p->d_od0))) return st;
-        const int L0 = march_config(p, p->nsys_build - p->N).L;
+        const bool fx = p->fx_imp.sys != nullptr;
+        const int L0 = fx ? p->fx_imp.sh.L : march_config(p, p->nsys_build - p->N).L;
         if ((st = factor_for(p, p->fs0L[lidx(L0)], L0, Vp, p->d_dg0, p->d_od0))) return st;
+        if (fx) LK(swr_launch_fx_prepare(p->fs0L[lidx(L0)], p->N, s));
         CK(cudaMemsetAsync(p->d_iface0, 0, sizeof(double2) * (nb + (size_t)p->ncols), s));
         // impulse marches only (the first N systems of the build list are the d marches)
         st = run_march(p, true, p->d_sys_build + p->N, p->nsys_build - p->N, nullptr,
@@ -2002,9 +2217,10 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
     if (p->autotune && !p->built) {
         // first build: measure the launch shapes of every march this plan makes
         const int k = march_kind(p, false);
-        if ((st = tune_march(p, k, false, p->d_sys_R, p->N, p->d_iface, p->d_V, p->d_dg, p->d_od)))
+        if (!p->fx_R.sys &&
+            (st = tune_march(p, k, false, p->d_sys_R, p->N, p->d_iface, p->d_V, p->d_dg, p->d_od)))
             return st;
-        if (k == MK_STATIC &&
+        if (k == MK_STATIC && !p->fx_build.sys &&
             (st = tune_march(p, k, false, p->d_sys_build, p->nsys_build, p->d_iface, p->d_V,
                              p->d_dg, p->d_od)))
             return st;
@@ -2016,13 +2232,20 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
                 Vp = p->d_Vbar;
             }
             if ((st = assemble(p, Vp, p->d_dg0, p->d_od0))) return st;
-            if ((st = tune_march(p, MK_STATIC, true, p->d_sys_build + p->N, p->nsys_build - p->N,
+            if (!p->fx_imp.sys && (st = tune_march(p, MK_STATIC, true, p->d_sys_build + p->N, p->nsys_build - p->N,
                                  p->d_iface, Vp, p->d_dg0, p->d_od0)))
                 return st;
         }
         // the probes wrote into d_iface; the build below starts the clock again
         CK(cudaMemsetAsync(p->d_iface, 0, sizeof(double2) * (nb + (size_t)p->ncols), s));
         CK(cudaEventRecord(p->ev[0], s));
+    }
+    for (auto& f : p->fx_stale) f = true;   // new factors; the build forms its own lists' form
+    if (p->fx_build.sys) p->fx_stale[lidx(p->fx_build.sh.L)] = false;
+    if (p->d.vkind == SWR_V_STATIC) {       // the chunk lengths this build factors
+        for (auto& f : p->fac_stale) f = true;
+        p->fac_stale[lidx(p->fx_build.sys ? p->fx_build.sh.L : march_config(p, p->nsys_build).L)] = false;
+        p->fac_stale[lidx(p->fx_R.sys ? p->fx_R.sh.L : march_config(p, p->N).L)] = false;
     }
     if (!p->built || !p->use_graph) {
         st = build_body(p, false);
@@ -2160,7 +2383,12 @@ swr_status swr_solve(swr_plan_t p, double* g_, int32_t g_is_initial, double* uT_
     if (p->superpose) {
         // u(T) from the build marches' states (the march is linear and time invariant);
         // the interface mismatch from w = L g + d and g
-        if (uT)
+        if (uT && p->fx_build.sys)
+            LK(swr_launch_superpose_fx(p->fsL[lidx(p->fx_build.sh.L)], p->d_urec, p->d_rec_base,
+                                       p->d_sys_final, p->d_subsys, p->N, p->d_n, p->d_goff,
+                                       p->d_tc, p->fx_build.d_scale, p->fx_build.d_shift, p->nt,
+                                       p->fx_build.d_bad, g, uT, s));
+        else if (uT)
             LK(swr_launch_superpose(p->d_urec, p->d_rec_base, p->d_sys_final, p->N, p->d_n,
                                     p->d_goff, p->d_tc, p->nmax, g, uT, s));
         if (p_toeplitz(p, p->d_iface + p->nb, g, p->d_iface, p->d_gtmp, 1))
@@ -2520,9 +2748,11 @@ swr_status swr_adjoint(swr_plan_t p, const double* ubar_, double* dJdV_, int32_t
             return st;
     }
     const MarchCfg cfg = march_config(p, N, MK_ADJ);
-    if (p->fsL[lidx(cfg.L)].L != cfg.L &&
-        (st = factor_for(p, p->fsL[lidx(cfg.L)], cfg.L, p->d_V, p->d_dg, p->d_od)))
-        return st;
+    if (p->fsL[lidx(cfg.L)].L != cfg.L || p->fac_stale[lidx(cfg.L)]) {
+        if ((st = factor_for(p, p->fsL[lidx(cfg.L)], cfg.L, p->d_V, p->d_dg, p->d_od))) return st;
+        p->fac_stale[lidx(cfg.L)] = false;
+        p->fx_stale[lidx(cfg.L)] = true;
+    }
     auto seg = [&](int mode, const double2* gin, int t0, int nrun, const double2* u0,
                    double2* uT) -> swr_status {
         SegArgs sa;

@@ -169,6 +169,16 @@ struct FactorSet {
     double2* tl_red = nullptr;
     int tl_rs = 32, tl_rl = 5;
     bool tl_ok = false;
+    // The same factors as fixed-point coefficients (swr_march_fx.cu; constant matrix, P + 1 <=
+    // kTlMaxSep), formed by swr_launch_fx_prepare.
+    struct FxSub* fx_sub = nullptr;   // [N] scales
+    unsigned long long* fx_mx = nullptr;   // maxima of the range analysis
+    int4* fx_rows = nullptr;          // [N][P+1][4 L + 13]
+    int4* fx_red = nullptr;           // [N][13][32]
+};
+// Scales of one subdomain's fixed-point march (shifts; see k_fx_bounds), bad: out of range.
+struct FxSub {
+    int s, s2, sd, kv, sr, kc, kr, bad;
 };
 constexpr int kTlMaxSep = 993;        // P + 1 <= 993: at most 32 super-separators
 constexpr int kTlMaxSepWide = 8161;   // P + 1 <= 8161: at most 256 super-separators
@@ -249,6 +259,43 @@ struct MarchArgs {
     // frev != 0 to walk them backwards (the adjoint's time-reversed march)
     int fstep0;
     int frev;
+    const int* only;      // march only the systems with only[sidx] != 0 (NULL: all)
+    int tstride;          // entries per trace (0: nt)
+};
+
+// Fixed-point march (swr_march_fx.cu): R right-hand sides per subdomain, grp[group][R] their
+// system indices (-1: none); u1 the states after step 1 (local node order, system q at soff[q]);
+// trace [nsys][2][nt] integer end traces; scale and bad per system.
+struct FxMarchArgs {
+    int nt, P, C, T, R;
+    const int* grp;
+    const MarchSys* sys;
+    const int* sub_tc;
+    const int* sub_P;
+    const int* sep_pos;
+    const unsigned char* clen;
+    const FxSub* fsub;
+    const int* sub_n;
+    const int4* rows;
+    const int4* red;
+    const long long* soff;
+    const double2* u1;
+    double2* urec;
+    double2* trace;
+    int* scale;
+    int* bad;
+    int* status;
+    int* tshift;          // [nsys][2][nt] scalings-down of the state before each trace entry
+    // driven marches (fin non-NULL): converted flux inputs [nsys][2][nt] (driven = 0: none),
+    // systems without input; uT and its first nodes for SYS_WRITE_UT
+    double2* fin;
+    int* tiny;
+    int driven;
+    double2* uT;
+    const int* sub_goff;
+};
+struct FxShape {
+    int L, C, T;
 };
 
 // One problem instance of a batched plan.  The instances' subdomains, interface
@@ -306,6 +353,21 @@ int swr_launch_march_tdep(const FactorSet& fs, MarchArgs a, const double* V, lon
                           double h, double kappa, double2 sig_ik, int ngroups, cudaStream_t s);
 int swr_march_smem_bytes(int T, int G, int stage_slots = 0);
 int swr_march_tl_smem_bytes(int T);
+
+// Fixed-point marches (swr_march_fx.cu).  swr_fx_shape: chunk length, CTAs per subdomain and
+// threads per right-hand side for ngroups subdomains of at most nmax nodes (false: none).
+bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out);
+int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s);
+int swr_launch_fx_start(const FactorSet& fs, FxMarchArgs a, int nsys, const double2* gin,
+                        double2 inv_ik, cudaStream_t s);
+int swr_launch_march_fx(const FactorSet& fs, FxMarchArgs a, int ngroups, cudaStream_t s);
+int swr_launch_fx_flux(const FxMarchArgs& a, int nsys, double2 two_sigma, const double2* gin,
+                       double2* gout, double2* vtrace, cudaStream_t s);
+int swr_launch_superpose_fx(const FactorSet& fs, const double2* urec, const long long* rec_base,
+                            const MarchSys* sys, const int3* subsys, int N, const int* sub_n,
+                            const int* sub_goff, const int* sub_tc, const int* scale,
+                            const int* shift, int ntmax, const int* bad, const double2* g,
+                            double2* uT, cudaStream_t s);
 
 // Interface algebra launchers (swr_krylov.cu)
 int swr_launch_toeplitz(int N, int nt, const double2* cols, const double2* x, const double2* add,

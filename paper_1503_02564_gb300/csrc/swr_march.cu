@@ -771,6 +771,10 @@ void swr_factor_free(FactorSet& fs) {
     cudaFree(fs.tl_pcr);
     cudaFree(fs.tl_aux);
     cudaFree(fs.tl_red);
+    cudaFree(fs.fx_sub);
+    cudaFree(fs.fx_mx);
+    cudaFree(fs.fx_rows);
+    cudaFree(fs.fx_red);
     fs = FactorSet();
 }
 
@@ -914,6 +918,10 @@ __global__ void __launch_bounds__((L == 16 || MODE == 2) ? 256 : 384, 1) k_march
     }
     bool valid = (p >= 0) && (sidx < a.nsys);
     if (ragged && valid && p > a.sub_P[a.sys[sidx].sub]) valid = false;   // the next system's
+    if (a.only) {   // a cluster holds one system: its CTAs leave together
+        valid = valid && a.only[sidx];
+        if (C > 1 ? !a.only[blockIdx.x / C] : !__syncthreads_or(valid)) return;
+    }
     const int rcbase = rbase - (g > 0 ? g : 0);   // ragged chunk slots: sum of P_j before
 
     auto SEP = [&](double2* arr, int ps) -> double2* {
@@ -1303,7 +1311,7 @@ __global__ void __launch_bounds__((L == 16 || MODE == 2) ? 256 : 384, 1) k_march
                     else if (s02v) o = cfma(a.two_c2, hsum[hs_l], o);
                     a.gout[(size_t)sy.out_a + a.t0 + t - 1] = o;
                 }
-                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 0) * nt + t - 1] = v;
+                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 0) * (a.tstride ? a.tstride : nt) + t - 1] = v;
             }
             if (p == Pj) {
                 if (hr) hist_r[ht0 + t] = v;
@@ -1314,7 +1322,7 @@ __global__ void __launch_bounds__((L == 16 || MODE == 2) ? 256 : 384, 1) k_march
                     else if (s02v) o = cfma(a.two_c2, hsum[hs_r], o);
                     a.gout[(size_t)sy.out_b + a.t0 + t - 1] = o;
                 }
-                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 1) * nt + t - 1] = v;
+                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 1) * (a.tstride ? a.tstride : nt) + t - 1] = v;
             }
         }
         if (rec_u && live) {   // u_t of this system in local node order
@@ -1423,6 +1431,7 @@ __global__ void __launch_bounds__((L == 16 || MODE == 2) ? 256 : 384, 1) k_march
     const int tid = threadIdx.x, lane = tid & 31, wl = tid >> 5;
     const int p = rank * T + tid;
     const int sidx = blockIdx.x / C;
+    if (a.only && !a.only[sidx]) return;   // one system per cluster: its CTAs leave together
     const double2 zero = make_double2(0.0, 0.0);
     const bool valid = (p <= P) && (sidx < a.nsys);
     MarchSys sy = {0, 0, 0, -1, -1, -1, -1, 0};
@@ -1715,7 +1724,7 @@ __global__ void __launch_bounds__((L == 16 || MODE == 2) ? 256 : 384, 1) k_march
                     else if (a.s02) o = cfma(a.two_c2, hsum[0], o);
                     a.gout[(size_t)sy.out_a + a.t0 + t - 1] = o;
                 }
-                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 0) * nt + t - 1] = v;
+                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 0) * (a.tstride ? a.tstride : nt) + t - 1] = v;
             }
             if (p == Pj) {
                 if (hr) hist_r[ht0 + t] = v;
@@ -1726,7 +1735,7 @@ __global__ void __launch_bounds__((L == 16 || MODE == 2) ? 256 : 384, 1) k_march
                     else if (a.s02) o = cfma(a.two_c2, hsum[1], o);
                     a.gout[(size_t)sy.out_b + a.t0 + t - 1] = o;
                 }
-                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 1) * nt + t - 1] = v;
+                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 1) * (a.tstride ? a.tstride : nt) + t - 1] = v;
             }
         }
         if (rec_u) {   // u_t of this system in local node order (streaming stores)
@@ -2082,12 +2091,12 @@ __global__ void __launch_bounds__(256, 1) k_march_tdep(const TdepArgs ta) {
             if (p == 0) {
                 if ((tcf & 1) && sy.out_a >= 0 && a.gout)
                     a.gout[(size_t)sy.out_a + t - 1] = csub(cmul(a.two_sigma, v), lin);
-                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 0) * nt + t - 1] = v;
+                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 0) * (a.tstride ? a.tstride : nt) + t - 1] = v;
             }
             if (p == Pj) {
                 if ((tcf & 2) && sy.out_b >= 0 && a.gout)
                     a.gout[(size_t)sy.out_b + t - 1] = csub(cmul(a.two_sigma, v), rin);
-                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 1) * nt + t - 1] = v;
+                if ((sy.flags & SYS_TRACE) && a.trace) a.trace[((size_t)sidx * 2 + 1) * (a.tstride ? a.tstride : nt) + t - 1] = v;
             }
         }
         SYNC();
