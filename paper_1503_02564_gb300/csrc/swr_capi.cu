@@ -130,6 +130,7 @@ struct swr_plan_s {
     double2* d_gtmp2 = nullptr;
     double2* d_trace = nullptr;    // N x 2 x nt
     MarchSys *d_sys_build = nullptr, *d_sys_R = nullptr, *d_sys_final = nullptr;
+    MarchSys* d_sys_L = nullptr;   // V(t,x), fixed-point marches: R from u0 = 0
     int nsys_build = 0;
     long long work_build = 0, work_build_imp = 0, work_R = 0;   // point-steps per launch
     int* d_status = nullptr;
@@ -166,13 +167,13 @@ struct swr_plan_s {
         int *d_scale = nullptr, *d_bad = nullptr;   // [nsys] scale of a system, marched in FP64
         int* d_shift = nullptr;          // [nsys][2][nt] its scalings-down, step by step
         double2* d_fin = nullptr;        // driven: [nsys][2][nt] converted inputs
-        int* d_tiny = nullptr;           // driven: [nsys] no input
         struct Launch {
             int start, count, T;
         };
         std::vector<Launch> launches;
     };
-    FxList fx_build, fx_imp, fx_d, fx_R, fx_final;
+    FxList fx_build, fx_imp, fx_d, fx_R, fx_final, fx_L;
+    bool fx_tdep = false;                // V(t,x): the per-step factors have a fixed-point form
     bool fx_stale[5] = {};               // fsL[] whose fixed-point form is older than its factors
     bool fac_stale[5] = {};              // fsL[] of another chunk length than the last build's
     int3* d_subsys = nullptr;            // per subdomain: its systems in the build list
@@ -633,18 +634,24 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     const int L = fl.sh.L;
     FactorSet& fs = zero_potential ? p->fs0L[lidx(L)] : p->fsL[lidx(L)];
     if (fs.L != L) return SWR_ERR_STATE;
-    const MarchCfg cfg = march_config(p, fl.nsys, MK_STATIC, L);
+    const bool steps = fs.nsteps > 1;   // per-step factors
+    const int kind = steps ? MK_TSTAT : MK_STATIC;
+    const MarchCfg cfg = steps ? march_config(p, fl.nsys, kind) : march_config(p, fl.nsys, kind, L);
     const int pi = prof_begin(p, 0, work);
     int rc = 0;
-    if (!zero_potential && p->fx_stale[lidx(L)]) {   // formed by the first march that needs it
+    if (!zero_potential && !steps && p->fx_stale[lidx(L)]) {   // formed by the first march that needs it
         rc = swr_launch_fx_prepare(fs, p->N, p->s);
         p->fx_stale[lidx(L)] = rc != 0;
     }
     SegArgs first, again;
     first.urec = p->d_fxu;
     first.tstride = p->nt;
+    if (p->cur_rev && steps) {   // time-reversed problem: last step's factors first
+        first.fstep0 = again.fstep0 = p->nt - 1;
+        first.frev = again.frev = 1;
+    }
     if (!rc)
-        rc = launch_cfg(p, cfg, MK_STATIC, zero_potential, fl.d_sys1, fl.nsys, gin, gout, nullptr,
+        rc = launch_cfg(p, cfg, kind, zero_potential, fl.d_sys1, fl.nsys, gin, gout, nullptr,
                         trace, u0, 1, first);
     FxMarchArgs a{};
     a.nt = p->nt;
@@ -664,8 +671,10 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     a.tshift = fl.d_shift;
     a.status = p->d_status;
     a.fin = fl.d_fin;
-    a.tiny = fl.d_tiny;
     a.driven = fl.driven && gin;
+    a.N = p->N;
+    a.fstep0 = first.fstep0;
+    a.frev = first.frev;
     if (!rc) rc = swr_launch_fx_start(fs, a, fl.nsys, gin, p->inv_ik, p->s);
     for (const auto& g : fl.launches) {
         a.grp = fl.d_grp + (size_t)g.start * fl.R;
@@ -675,8 +684,8 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     if (!rc) rc = swr_launch_fx_flux(a, fl.nsys, p->two_sigma, gin, gout, trace, p->s);
     again.only = fl.d_bad;
     if (!rc)
-        rc = launch_cfg(p, cfg, MK_STATIC, zero_potential, fl.sys, fl.nsys, gin, gout, uT, trace,
-                        u0, p->nt, again);
+        rc = launch_cfg(p, cfg, kind, zero_potential, fl.sys, fl.nsys, gin, gout, uT, trace, u0,
+                        p->nt, again);
     prof_end(p, pi);
     return rc ? launch_fail("march (fixed point)", __LINE__) : SWR_OK;
 }
@@ -686,8 +695,9 @@ swr_status run_march(swr_plan_t p, bool zero_potential, const MarchSys* d_sys, i
                      const double2* gin, double2* gout, double2* uT, double2* trace,
                      const double2* u0, long long work, double2* vrec = nullptr) {
     const int kind = march_kind(p, zero_potential);
-    for (const auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final})
-        if (kind == MK_STATIC && fl->sys && fl->sys == d_sys && fl->nsys == nsys && !vrec)
+    for (const auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final, &p->fx_L})
+        if ((kind == MK_STATIC || (kind == MK_TSTAT && p->fx_tdep)) && fl->sys && fl->sys == d_sys &&
+            fl->nsys == nsys && !vrec)
             return run_march_fx(p, zero_potential, *fl, gin, gout, uT, trace, u0, work);
     const MarchCfg cfg = march_config(p, nsys, kind);
     const int pi = prof_begin(p, kind == MK_NL ? 3 : 0, work);
@@ -739,13 +749,15 @@ swr_status factor_for(swr_plan_t p, FactorSet& fs, int L, const double* V, doubl
 swr_status factor_steps_for(swr_plan_t p, FactorSet& fs, int L, int nsteps);
 
 swr_status tune_march(swr_plan_t p, int kind, bool zero_potential, const MarchSys* d_sys,
-                      int nsys, double2* gout, const double* V, double2* dg, double2* od) {
+                      int nsys, double2* gout, const double* V, double2* dg, double2* od,
+                      int onlyL = 0) {
     if (!p->autotune || nsys <= 0 || (p->long_march && kind == MK_STATIC)) return SWR_OK;
     for (const auto& t : p->tuned)
         if (t[0] == kind && t[1] == nsys) return SWR_OK;
-    const MarchCfg guess = march_config(p, nsys, kind);
+    const MarchCfg guess = march_config(p, nsys, kind, onlyL);
     std::vector<int> Ls;
-    if (kind == MK_TDEP) Ls = {4};
+    if (onlyL) Ls = {onlyL};
+    else if (kind == MK_TDEP) Ls = {4};
     else if (kind == MK_NL && (p->forceL == 2 || p->forceL == 4 || p->forceL == 8))
         Ls = {p->forceL};
     else if (kind == MK_NL) Ls = {8, 4, 2};   // 2: two warps per sub-partition for short systems
@@ -879,6 +891,8 @@ swr_status factor_steps_for(swr_plan_t p, FactorSet& fs, int L, int nsteps) {
         if (swr_factor_alloc(fs, p->N, L, chunks_for(p->nmax, L), p->s, nsteps, p->ntot) != 0)
             return SWR_ERR_NOMEM;
     }
+    if (p->fx_tdep && nsteps == p->nt && !fs.fx_steps && swr_fx_alloc_steps(fs, p->N) != 0)
+        p->fx_tdep = false;
     if (swr_launch_factor_steps(fs, p->N, p->d_n, p->d_goff, p->d_loff, p->d_tc, p->nmax, p->d_V,
                                 p->nx, p->h, p->d.dt, p->sigma0, p->inv_ik, p->d_status,
                                 p->s) != 0) {
@@ -1025,7 +1039,6 @@ swr_status fx_list(swr_plan_t p, swr_plan_s::FxList& fl, const MarchSys* sys, co
     if (!st) st = dalloc(&fl.d_bad, (size_t)nsys);
     if (!st) st = dalloc(&fl.d_shift, (size_t)nsys * 2 * p->nt);
     if (!st && driven) st = dalloc(&fl.d_fin, (size_t)nsys * 2 * p->nt);
-    if (!st && driven) st = dalloc(&fl.d_tiny, (size_t)nsys);
     if (!st && !p->d_fxu) {   // shared by the lists: the longest one is set up first
         st = dalloc(&p->d_fxu, (size_t)tot);
         if (!st) st = dalloc(&p->d_fxtrace, (size_t)nsys * 2 * p->nt);
@@ -1143,6 +1156,14 @@ swr_status apply_A(swr_plan_t p, const double2* x, double2* y) {
         const int rc = p_toeplitz(p, p->d_iface + p->nb, x, nullptr, y, 0);
         prof_end(p, pi);
         return rc ? SWR_ERR_UNSUPPORTED : SWR_OK;
+    }
+    if (p->fx_tdep && march_kind(p, false) == MK_TSTAT) {
+        // L x is R x from u0 = 0: the fixed-point march then has the scale of x, where R x - d
+        // would keep the absolute error of the states that u0 brings
+        swr_status st = run_march(p, false, p->d_sys_L, p->N, x, y, nullptr, nullptr, p->d_u0, p->work_R);
+        if (st) return st;
+        LK(swr_launch_axpby(y, x, n, make_double2(-1.0, 0.0), make_double2(1.0, 0.0), p->s));
+        return SWR_OK;
     }
     // matrix-free: y = x - R x + d   (Algorithm 2)
     const double2* u0 = p->cur_u0 ? p->cur_u0 : p->d_u0;
@@ -1652,10 +1673,10 @@ void swr_destroy(swr_plan_t p) {
     cudaFree(p->d_u0); cudaFree(p->d_V); cudaFree(p->d_Vbar); cudaFree(p->d_iface); cudaFree(p->d_iface0);
     cudaFree(p->d_lag0); cudaFree(p->d_lag0_0); cudaFree(p->d_hist); cudaFree(p->d_gtmp);
     cudaFree(p->d_gtmp2); cudaFree(p->d_trace);
-    cudaFree(p->d_sys_build); cudaFree(p->d_sys_R); cudaFree(p->d_sys_final);
+    cudaFree(p->d_sys_build); cudaFree(p->d_sys_R); cudaFree(p->d_sys_final); cudaFree(p->d_sys_L);
     cudaFree(p->d_status); cudaFree(p->d_scal); cudaFree(p->d_pit);
     cudaFree(p->d_urec); cudaFree(p->d_rec_base);
-    for (auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final}) {
+    for (auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final, &p->fx_L}) {
         cudaFree(fl->d_sys1);
         cudaFree(fl->d_grp);
         cudaFree(fl->d_soff);
@@ -1663,7 +1684,6 @@ void swr_destroy(swr_plan_t p) {
         cudaFree(fl->d_bad);
         cudaFree(fl->d_shift);
         cudaFree(fl->d_fin);
-        cudaFree(fl->d_tiny);
     }
     cudaFree(p->d_subsys); cudaFree(p->d_fxu); cudaFree(p->d_fxtrace);
     cudaFree(p->d_W); cudaFree(p->d_spec); cudaFree(p->d_spec0); cudaFree(p->d_Gw);
@@ -1933,9 +1953,11 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
                     swr_fx_shape(p->nmax, p->N, fxR, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fxs);
     // the marches of one system per subdomain (R g, final, the adjoint's d)
     FxShape fx1{};
-    const bool fx_one = d->vkind == SWR_V_STATIC && d->tc == SWR_TC_ROBIN && !is_long &&
+    const bool fx_one = d->vkind != SWR_V_NONLINEAR && d->tc == SWR_TC_ROBIN && !is_long &&
                         p->two_level && p->nt >= 16 &&
-                        swr_fx_shape(p->nmax, p->N, 1, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fx1);
+                        (d->vkind != SWR_V_TIME || p->tune.tdep_precomp >= 0) &&
+                        swr_fx_shape(p->nmax, p->N, 1, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fx1,
+                                     d->vkind == SWR_V_TIME);
     p->rec_n.resize(p->N);
     for (int j = 0; j < p->N; ++j)   // chunk-element order: (L + 1) rows of P_j + 1
         p->rec_n[j] = fx && fxR == 3 ? (fxs.L + 1) * (chunks_for(p->n[j], fxs.L) + 1) : p->n[j];
@@ -1987,7 +2009,7 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
                              p->nsys_build - p->N, 2, sh);
         }
         if (!st && fx_one)
-            st = fx_list(p, p->fx_d, p->d_sys_build, vb.data(), p->N, 1, fx1);
+            st = fx_list(p, p->fx_d, p->d_sys_build, vb.data(), p->N, 1, fx1, d->vkind == SWR_V_TIME);
     }
     if (!st && is_long) {
         // a subdomain longer than one cluster can hold (16 CTAs x 256 chunks of 16 nodes):
@@ -2063,6 +2085,11 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
     if (!st && fx_one) {
         auto vr = apply_systems(p, 0), vf = apply_systems(p, SYS_WRITE_UT | SYS_TRACE);
         st = fx_list(p, p->fx_R, p->d_sys_R, vr.data(), p->N, 1, fx1, true);
+        if (!st && d->vkind == SWR_V_TIME) {
+            auto vl = apply_systems(p, SYS_ZERO_U0);
+            st = upload_systems(&p->d_sys_L, vl, p);
+            if (!st) st = fx_list(p, p->fx_L, p->d_sys_L, vl.data(), p->N, 1, fx1, true);
+        }
         if (!st && !p->superpose)
             st = fx_list(p, p->fx_final, p->d_sys_final, vf.data(), p->N, 1, fx1, true);
     }
@@ -2213,12 +2240,26 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
             on = need <= fr / 2;
         }
         p->tdep_pre = on ? 1 : 0;
+        if (on && p->fx_R.sys) {
+            // the fixed-point form beside them: another set of the same size, within a quarter
+            // of the free memory
+            size_t fr = 0, tot = 0;
+            CK(cudaMemGetInfo(&fr, &tot));
+            const int L = p->fx_R.sh.L, P = chunks_for(p->nmax, L);
+            const size_t fac = (size_t)p->nt * swr_factor_step_bytes(p->N, L, P);
+            p->fx_tdep = fac <= fr / 2 && (size_t)p->nt * swr_fx_step_bytes(p->N, L, P) <= fr / 4;
+            if (p->fx_tdep && !p->autotune) {   // one chunk length for both forms
+                const MarchCfg c = march_config(p, p->N, MK_TSTAT, L);
+                p->tuned.push_back({MK_TSTAT, p->N, c.L, c.C, c.G, c.T, c.ngroups, c.ragged});
+            }
+        }
     }
     if (p->autotune && !p->built) {
         // first build: measure the launch shapes of every march this plan makes
         const int k = march_kind(p, false);
-        if (!p->fx_R.sys &&
-            (st = tune_march(p, k, false, p->d_sys_R, p->N, p->d_iface, p->d_V, p->d_dg, p->d_od)))
+        if ((k != MK_STATIC || !p->fx_R.sys) &&
+            (st = tune_march(p, k, false, p->d_sys_R, p->N, p->d_iface, p->d_V, p->d_dg, p->d_od,
+                             p->fx_tdep ? p->fx_R.sh.L : 0)))
             return st;
         if (k == MK_STATIC && !p->fx_build.sys &&
             (st = tune_march(p, k, false, p->d_sys_build, p->nsys_build, p->d_iface, p->d_V,

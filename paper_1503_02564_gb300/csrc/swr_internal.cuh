@@ -175,6 +175,8 @@ struct FactorSet {
     unsigned long long* fx_mx = nullptr;   // maxima of the range analysis
     int4* fx_rows = nullptr;          // [N][P+1][4 L + 13]
     int4* fx_red = nullptr;           // [N][13][32]
+    // nsteps > 1 (swr_fx_alloc_steps): fx_sub, fx_rows and fx_red hold one copy per step
+    bool fx_steps = false;
 };
 // Scales of one subdomain's fixed-point march (shifts; see k_fx_bounds), bad: out of range.
 struct FxSub {
@@ -286,13 +288,14 @@ struct FxMarchArgs {
     int* bad;
     int* status;
     int* tshift;          // [nsys][2][nt] scalings-down of the state before each trace entry
-    // driven marches (fin non-NULL): converted flux inputs [nsys][2][nt] (driven = 0: none),
-    // systems without input; uT and its first nodes for SYS_WRITE_UT
+    // driven marches (fin non-NULL): converted flux inputs [nsys][2][nt] (driven = 0: none); uT
+    // and its first nodes for SYS_WRITE_UT
     double2* fin;
-    int* tiny;
     int driven;
     double2* uT;
     const int* sub_goff;
+    // per-step factors: subdomains N, the step-1 set and the direction of the walk
+    int stream, N, fstep0, frev;
 };
 struct FxShape {
     int L, C, T;
@@ -356,8 +359,14 @@ int swr_march_tl_smem_bytes(int T);
 
 // Fixed-point marches (swr_march_fx.cu).  swr_fx_shape: chunk length, CTAs per subdomain and
 // threads per right-hand side for ngroups subdomains of at most nmax nodes (false: none).
-bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out);
-int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s);
+bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out,
+                  bool stream = false);
+// (nb steps from t0 on, for per-step factors)
+int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0 = 0, int nb = 1);
+// Room for the fixed-point form of per-step factors (nsteps > 1), filled by
+// swr_launch_factor_steps: 0, -1 (no memory) or -2 (too many separators).
+size_t swr_fx_step_bytes(int N, int L, int P);
+int swr_fx_alloc_steps(FactorSet& fs, int N);
 int swr_launch_fx_start(const FactorSet& fs, FxMarchArgs a, int nsys, const double2* gin,
                         double2 inv_ik, cudaStream_t s);
 int swr_launch_march_fx(const FactorSet& fs, FxMarchArgs a, int ngroups, cudaStream_t s);

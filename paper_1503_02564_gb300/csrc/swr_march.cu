@@ -57,10 +57,19 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // P1 interpolant of W), scaled by 1/(i kappa).  dg[loff_j + i] is the diagonal,
 // od[loff_j + i] the coupling of local nodes i and i+1.
 // ---------------------------------------------------------------------------
+// The grid's constants come from the host: an FP64 division in every thread (seven of them)
+// made this kernel 11.8 us per 1000 nodes-steps of V(t,x) tables, against 3.2 us.
+struct AsmConsts {
+    double h3, ih, h12, tdt, e_im;   // h/3, 1/h, h/12, 2/dt, (2/dt)(h/6)
+};
+static AsmConsts asm_consts(double h, double dt) {
+    return AsmConsts{h / 3.0, 1.0 / h, h / 12.0, 2.0 / dt, 2.0 / dt * (h / 6.0)};
+}
+
 __global__ void k_assemble_static(const double* __restrict__ V, long long vstride,
                                   const int* __restrict__ n_, const int* __restrict__ goff_,
                                   const int* __restrict__ loff_, const int* __restrict__ tc_,
-                                  double h, double dt, double2 sigma0, double2 inv_ik,
+                                  AsmConsts cst, double2 sigma0, double2 inv_ik,
                                   double2* __restrict__ dg, double2* __restrict__ od,
                                   long long ldd, const double2* __restrict__ kap = nullptr,
                                   int kstride = 0) {
@@ -81,24 +90,24 @@ __global__ void k_assemble_static(const double* __restrict__ V, long long vstrid
     double md = 0.0, sd = 0.0, wd = 0.0;
     if (i > 0) {
         const double Wm = W(g - 1);
-        md += h / 3.0;
-        sd += 1.0 / h;
-        wd += h / 12.0 * (Wm + 3.0 * W0);
+        md += cst.h3;
+        sd += cst.ih;
+        wd += cst.h12 * (Wm + 3.0 * W0);
     }
     if (i < n - 1) {
         const double Wp = W(g + 1);
-        md += h / 3.0;
-        sd += 1.0 / h;
-        wd += h / 12.0 * (3.0 * W0 + Wp);
+        md += cst.h3;
+        sd += cst.ih;
+        wd += cst.h12 * (3.0 * W0 + Wp);
     }
-    double2 D = make_double2(-sd + wd, 2.0 / dt * md);
+    double2 D = make_double2(-sd + wd, cst.tdt * md);
     // the end's boundary entry: sigma0, or the lag-0 entry of its own kernel
     if (i == 0 && (tc & 1)) D = csub(D, kap ? kap[(size_t)(2 * j + 0) * kstride] : sigma0);
     if (i == n - 1 && (tc & 2)) D = csub(D, kap ? kap[(size_t)(2 * j + 1) * kstride] : sigma0);
     dg[lo] = cmul(D, inv_ik);
     if (i < n - 1) {
         const double Wp = W(g + 1);
-        const double2 E = make_double2(1.0 / h + h / 12.0 * (W0 + Wp), 2.0 / dt * (h / 6.0));
+        const double2 E = make_double2(cst.ih + cst.h12 * (W0 + Wp), cst.e_im);
         od[lo] = cmul(E, inv_ik);
     } else {
         od[lo] = make_double2(0.0, 0.0);
@@ -197,7 +206,7 @@ int swr_launch_assemble_static(const double* V, int N, const int* d_n, const int
                                double2 sigma0, double2 inv_ik, double2* dg, double2* od,
                                cudaStream_t s, const double2* kap, int kstride) {
     dim3 grid((nmax + 255) / 256, N);
-    k_assemble_static<<<grid, 256, 0, s>>>(V, 0, d_n, d_goff, d_loff, d_tc, h, dt, sigma0, inv_ik,
+    k_assemble_static<<<grid, 256, 0, s>>>(V, 0, d_n, d_goff, d_loff, d_tc, asm_consts(h, dt), sigma0, inv_ik,
                                            dg, od, 0, kap, kstride);
     swr_count_launch(1);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -496,7 +505,7 @@ __global__ void __launch_bounds__(1024, 1) k_factor_two_level(
     const double2* __restrict__ od, const int* __restrict__ sub_P,
     const int* __restrict__ sep_pos, const double2* __restrict__ tips,
     double2* __restrict__ tl_pcr, double2* __restrict__ tl_aux, double2* __restrict__ tl_red,
-    int RS, int RL, int* status) {
+    int RS, int RL, int* status, long long ldd) {
     // per super-separator q: its row (lo, dd, up); per super-chunk q: the spikes at its
     // first member (af, bf) and last member (al, bl); wide reduced PCR: rows L, D, U
     extern __shared__ double2 fsm[];
@@ -507,6 +516,15 @@ __global__ void __launch_bounds__(1024, 1) k_factor_two_level(
     const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5, nw = blockDim.x >> 5;
     const int Pj = sub_P[j];
     const int S = P + 1;
+    {   // batch entry z (per-step factorisations): its own matrix and tips, its own outputs
+        const size_t z = blockIdx.y;
+        dg += z * ldd;
+        od += z * ldd;
+        tips += z * N * P * 4;
+        tl_pcr += z * N * 10 * S;
+        tl_aux += z * N * 3 * S;
+        tl_red += z * N * (2 * RL + 3) * RS;
+    }
     const int Q = (Pj + 31) / 32;
     const double2 zero = make_double2(0.0, 0.0), one = make_double2(1.0, 0.0);
     const double2* T = tips + (size_t)j * P * 4;
@@ -694,7 +712,7 @@ int swr_launch_factor_tl(FactorSet& fs, int N, const int* d_loff, const double2*
     const int threads = std::min(1024, std::max(RS, ((S + 31) / 32) * 32));
     k_factor_two_level<<<N, threads, sizeof(double2) * 13 * RS, s>>>(
         N, fs.P, d_loff, dg, od, fs.sub_P, fs.sep_pos, fs.tips, fs.tl_pcr, fs.tl_aux, fs.tl_red,
-        RS, RL, status);
+        RS, RL, status, 0);
     swr_count_launch(1);
     if (cudaGetLastError() != cudaSuccess) return -1;
     fs.tl_ok = true;
@@ -837,13 +855,25 @@ int swr_launch_factor_steps(FactorSet& fs, int N, const int* d_n, const int* d_g
         const int nb = std::min(fs.batch, fs.nsteps - t0);
         dim3 grid((nmax + 255) / 256, N, nb);
         k_assemble_static<<<grid, 256, 0, s>>>(V + (size_t)t0 * vstride, vstride, d_n, d_goff,
-                                               d_loff, d_tc, h, dt, sigma0, inv_ik, fs.dgb, fs.odb,
+                                               d_loff, d_tc, asm_consts(h, dt), sigma0, inv_ik, fs.dgb, fs.odb,
                                                fs.ldd);
         swr_count_launch(1);
         if (cudaGetLastError() != cudaSuccess) return -1;
-        const int rc = launch_factor_batch(fs, N, d_n, d_loff, fs.dgb, fs.odb, fs.ldd, t0, nb,
-                                           status, s);
+        int rc = launch_factor_batch(fs, N, d_n, d_loff, fs.dgb, fs.odb, fs.ldd, t0, nb, status, s);
         if (rc) return rc;
+        if (fs.fx_steps) {   // the batch in fixed point, from its two-level separator data
+            const int S = fs.P + 1;
+            if (S > 32) {
+                k_factor_two_level<<<dim3(N, nb), std::max(32, ((S + 31) / 32) * 32),
+                                     sizeof(double2) * 13 * 32, s>>>(
+                    N, fs.P, d_loff, fs.dgb, fs.odb, fs.sub_P, fs.sep_pos, fs.tips, fs.tl_pcr,
+                    fs.tl_aux, fs.tl_red, 32, 5, status, fs.ldd);
+                swr_count_launch(1);
+                if (cudaGetLastError() != cudaSuccess) return -1;
+            }
+            rc = swr_launch_fx_prepare(fs, N, s, t0, nb);
+            if (rc) return rc;
+        }
     }
     return 0;
 }

@@ -65,7 +65,12 @@ constexpr int kFxSlack = 1;
 
 size_t swr_fx_bounds_bytes(int N) { return sizeof(unsigned long long) * B_N * (size_t)N; }
 
-__device__ __forceinline__ double cabs_(double2 a) { return sqrt(fma(a.x, a.x, a.y * a.y)); }
+// |a| from above, at most 8 % over: sqrt(m^2 + n^2) <= m + (sqrt(2) - 1) n for n <= m (a square
+// root is some twenty FP64 instructions)
+__device__ __forceinline__ double cabs_(double2 a) {
+    const double x = fabs(a.x), y = fabs(a.y);
+    return x > y ? fma(0.41422, y, x) : fma(0.41422, x, y);
+}
 
 // maxima of subdomain j's coefficients and absolute recurrences into mx[j]; threads over
 // chunks / separators p of one tile
@@ -74,10 +79,21 @@ __global__ void __launch_bounds__(64) k_fx_bounds(
     const unsigned char* __restrict__ clen, const double2* __restrict__ fac,
     const double2* __restrict__ sep, const double2* __restrict__ pcr,
     const double2* __restrict__ tl_pcr, const double2* __restrict__ tl_aux,
-    const double2* __restrict__ tl_red, unsigned long long* __restrict__ mx) {
+    const double2* __restrict__ tl_red, unsigned long long* __restrict__ mx, long long fstride,
+    long long sstride, long long pstride) {
     __shared__ unsigned long long sm[B_N];
     const int j = blockIdx.y, S = P + 1, p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int Pj = sub_P[j], Q = (Pj + 31) / 32;
+    const int Pj = sub_P[j], Q = (Pj + 31) / 32, N = gridDim.y;
+    {   // batch entry z (per-step factors)
+        const size_t z = blockIdx.z;
+        fac += z * fstride;
+        sep += z * sstride;
+        pcr += z * pstride;
+        tl_pcr += z * N * 10 * S;
+        tl_aux += z * N * 3 * S;
+        tl_red += z * N * 13 * 32;
+        mx += z * N * B_N;
+    }
     for (int k = threadIdx.x; k < B_N; k += blockDim.x) sm[k] = 0;
     __syncthreads();
     // |x| of a finite or NaN double orders as an integer (NaN above everything)
@@ -156,7 +172,7 @@ __device__ __forceinline__ FxSub fx_sub(const unsigned long long* mx, int& eb, i
             g2 *= 1.0 + get(B_RG + k);
             bad |= get(B_PG + k) > 2.6 || get(B_RG + k) > 2.6;
         }
-        bad |= get(B_CO) > 1.0 || get(B_AX) > 2.6 || get(B_Y) > 4.0;
+        bad |= get(B_CO) > 1.1 || get(B_AX) > 2.6 || get(B_Y) > 4.0;
         // a separator's row: its stencil and a flux, the two chunks' parts
         const double d0 = 2.0 * kFxF + get(B_D) + get(B_CZ);
         f.s = max(0, fx_clog2(fmax(get(B_Z), 1.0)) - 2);
@@ -192,9 +208,23 @@ __global__ void __launch_bounds__(64) k_fx_convert(
     const double2* __restrict__ sep, const double2* __restrict__ pcr,
     const double2* __restrict__ tl_pcr, const double2* __restrict__ tl_aux,
     const double2* __restrict__ tl_red, const unsigned long long* __restrict__ mx,
-    FxSub* __restrict__ fsub, int4* __restrict__ rows, int4* __restrict__ red) {
+    FxSub* __restrict__ fsub, int4* __restrict__ rows, int4* __restrict__ red, long long fstride,
+    long long sstride, long long pstride) {
     const int j = blockIdx.y, S = P + 1, p = blockIdx.x * blockDim.x + threadIdx.x;
-    const int Pj = sub_P[j], Q = (Pj + 31) / 32;
+    const int Pj = sub_P[j], Q = (Pj + 31) / 32, N = gridDim.y;
+    {   // batch entry z (per-step factors)
+        const size_t z = blockIdx.z;
+        fac += z * fstride;
+        sep += z * sstride;
+        pcr += z * pstride;
+        tl_pcr += z * N * 10 * S;
+        tl_aux += z * N * 3 * S;
+        tl_red += z * N * 13 * 32;
+        mx += z * N * B_N;
+        fsub += z * N;
+        rows += z * N * S * (4 * L + 13);
+        red += z * N * 13 * 32;
+    }
     int eb, er, eC;
     const FxSub f = fx_sub(mx + (size_t)j * B_N, eb, er, eC);
     if (blockIdx.x == 0 && threadIdx.x == 0) fsub[j] = f;
@@ -247,27 +277,66 @@ __global__ void __launch_bounds__(64) k_fx_convert(
     }
 }
 
-int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s) {
-    if (fs.nsteps != 1) return -2;
-    const int S = fs.P + 1, one = S <= 32;
-    if (!one && (!fs.tl_ok || fs.tl_rs != 32)) return -2;
-    if (!fs.fx_sub) {
-        bool ok = cudaMalloc(&fs.fx_sub, sizeof(FxSub) * N) == cudaSuccess;
-        ok &= cudaMalloc(&fs.fx_mx, swr_fx_bounds_bytes(N)) == cudaSuccess;
-        ok &= cudaMalloc(&fs.fx_rows, sizeof(int4) * (size_t)N * S * (4 * fs.L + 13)) == cudaSuccess;
-        ok &= cudaMalloc(&fs.fx_red, sizeof(int4) * (size_t)N * 13 * 32) == cudaSuccess;
+static bool fx_alloc(FactorSet& fs, int N, int nsteps, int batch) {
+    const size_t S = fs.P + 1, ns = nsteps;
+    bool ok = cudaMalloc(&fs.fx_sub, sizeof(FxSub) * N * ns) == cudaSuccess;
+    ok &= cudaMalloc(&fs.fx_mx, swr_fx_bounds_bytes(N) * batch) == cudaSuccess;
+    ok &= cudaMalloc(&fs.fx_rows, sizeof(int4) * ns * N * S * (4 * fs.L + 13)) == cudaSuccess;
+    ok &= cudaMalloc(&fs.fx_red, sizeof(int4) * ns * N * 13 * 32) == cudaSuccess;
+    if (!ok) {
+        cudaGetLastError();
+        cudaFree(fs.fx_sub);
+        cudaFree(fs.fx_mx);
+        cudaFree(fs.fx_rows);
+        cudaFree(fs.fx_red);
+        fs.fx_sub = nullptr;
+        fs.fx_mx = nullptr;
+        fs.fx_rows = fs.fx_red = nullptr;
+    }
+    return ok;
+}
+
+size_t swr_fx_step_bytes(int N, int L, int P) {
+    return sizeof(int4) * N * ((size_t)(P + 1) * (4 * L + 13) + 13 * 32) + sizeof(FxSub) * N;
+}
+
+int swr_fx_alloc_steps(FactorSet& fs, int N) {
+    const size_t S = fs.P + 1;
+    if (fs.nsteps < 2 || S >= kTlMaxSep) return -2;
+    if (fs.fx_steps) return 0;
+    if (!fs.tl_pcr && S > 32) {   // two-level data of one batch
+        const size_t nb = fs.batch;
+        bool ok = cudaMalloc(&fs.tl_pcr, sizeof(double2) * nb * N * 10 * S) == cudaSuccess;
+        ok &= cudaMalloc(&fs.tl_aux, sizeof(double2) * nb * N * 3 * S) == cudaSuccess;
+        ok &= cudaMalloc(&fs.tl_red, sizeof(double2) * nb * N * 13 * 32) == cudaSuccess;
         if (!ok) {
             cudaGetLastError();
             return -1;
         }
     }
-    const dim3 grid((S + 63) / 64, N);
-    if (cudaMemsetAsync(fs.fx_mx, 0, swr_fx_bounds_bytes(N), s) != cudaSuccess) return -1;
-    k_fx_bounds<<<grid, 64, 0, s>>>(fs.L, fs.P, fs.levels, one, fs.sub_P, fs.clen, fs.fac, fs.sep,
-                                    fs.pcr, fs.tl_pcr, fs.tl_aux, fs.tl_red, fs.fx_mx);
-    k_fx_convert<<<grid, 64, 0, s>>>(fs.L, fs.P, fs.levels, one, fs.sub_P, fs.clen, fs.fac, fs.sep,
-                                     fs.pcr, fs.tl_pcr, fs.tl_aux, fs.tl_red, fs.fx_mx, fs.fx_sub,
-                                     fs.fx_rows, fs.fx_red);
+    if (!fx_alloc(fs, N, fs.nsteps, fs.batch)) return -1;
+    fs.fx_steps = true;
+    return 0;
+}
+
+int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0, int nb) {
+    const int S = fs.P + 1, one = S <= 32;
+    if (fs.nsteps > 1 ? !fs.fx_steps : (!one && (!fs.tl_ok || fs.tl_rs != 32))) return -2;
+    if (!fs.fx_sub && !fx_alloc(fs, N, 1, 1)) return -1;
+    const dim3 grid((S + 63) / 64, N, nb);
+    if (cudaMemsetAsync(fs.fx_mx, 0, swr_fx_bounds_bytes(N) * nb, s) != cudaSuccess) return -1;
+    const double2* fac = fs.fac + (size_t)t0 * fs.fstride;
+    const double2* sep = fs.sep + (size_t)t0 * fs.sstride;
+    const double2* pcr = fs.pcr + (size_t)t0 * fs.pstride;
+    k_fx_bounds<<<grid, 64, 0, s>>>(fs.L, fs.P, fs.levels, one, fs.sub_P, fs.clen, fac, sep, pcr,
+                                    fs.tl_pcr, fs.tl_aux, fs.tl_red, fs.fx_mx, fs.fstride,
+                                    fs.sstride, fs.pstride);
+    k_fx_convert<<<grid, 64, 0, s>>>(fs.L, fs.P, fs.levels, one, fs.sub_P, fs.clen, fac, sep, pcr,
+                                     fs.tl_pcr, fs.tl_aux, fs.tl_red, fs.fx_mx,
+                                     fs.fx_sub + (size_t)t0 * N,
+                                     fs.fx_rows + (size_t)t0 * N * S * (4 * fs.L + 13),
+                                     fs.fx_red + (size_t)t0 * N * 13 * 32, fs.fstride, fs.sstride,
+                                     fs.pstride);
     swr_count_launch(2);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -305,10 +374,15 @@ __global__ void __launch_bounds__(256) k_fx_start(const FxMarchArgs a, const dou
             f = max(f, (unsigned long long)__double_as_longlong(fabs(v.y)));
         }
     atomicMax(&mf, f);
-    __syncthreads();
+    bool out = false;   // per-step factors: any step's out of range
+    if (a.stream)
+        for (int t = threadIdx.x; t < sy.nt; t += blockDim.x)
+            out |= a.fsub[(size_t)(a.fstep0 + (a.frev ? -t : t)) * a.N + j].bad != 0;
+    out = __syncthreads_or(out);
     if (threadIdx.x == 0) {
         double top = __longlong_as_double((long long)mx), tf = __longlong_as_double((long long)mf);
-        int sc = 0, b = a.fsub[j].bad;
+        int sc = 0, b = a.stream ? 0 : a.fsub[j].bad;
+        b |= out;
         for (double v : {top, tf}) b |= !isfinite(v) || v > 1e250;
         if (top < 1e-280) top = 0.0;   // far tails of a packet: marched as zero
         if (tf < 1e-280) tf = 0.0;
@@ -321,7 +395,6 @@ __global__ void __launch_bounds__(256) k_fx_start(const FxMarchArgs a, const dou
         }
         a.scale[q] = ssc = sc;
         a.bad[q] = sbad = b;
-        if (a.fin) a.tiny[q] = tf > 0.0 ? 0 : 1;   // no input: the traces decide (k_fx_flux)
     }
     __syncthreads();
     if (!a.fin || sbad || !gin) return;
@@ -379,17 +452,21 @@ __device__ __forceinline__ bool fx_wait(unsigned mbar, unsigned parity) {
     return false;
 }
 
-template <int L, bool ONE, bool FLUX>
-__global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 ? 512 : 384), 1)
+template <int L, bool ONE, bool FLUX, bool STREAM>
+__global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384), 1)
     k_march_fx(const FxMarchArgs a) {
     constexpr int ROW = 4 * L + 13;
     constexpr int KT = FLUX ? 24 : 25;   // the trigger is 2^(32 + KT)
     extern __shared__ int4 fsm[];
     const int T = ONE ? 32 : a.T, C = ONE ? 1 : a.C, R = a.R, P = a.P, S = P + 1;
-    int4* srd = fsm + ROW * T;                                       // [13][32] reduced system
-    FxC* sA = reinterpret_cast<FxC*>(srd + (ONE ? 0 : 13 * 32));     // [2][R][kFxSlots]
-    FxC* sB = sA + 2 * R * kFxSlots;
-    unsigned long long* mbar = reinterpret_cast<unsigned long long*>(sB + 2 * R * kFxSlots);   // [2][R]
+    const int RD = ONE ? 0 : 13 * 32;
+    const int BUF = ROW * T + RD;         // rows, then the reduced system [13][32]; STREAM: two
+    const int4* srd = fsm + ROW * T;
+    FxC* sA = reinterpret_cast<FxC*>(fsm + (STREAM ? 2 : 1) * BUF);  // [2][R][kFxSlots]
+    FxC* sB = sA + (ONE ? 0 : 2 * R * kFxSlots);
+    unsigned long long* mbar =
+        reinterpret_cast<unsigned long long*>(sB + (ONE ? 0 : 2 * R * kFxSlots));   // [2][R]
+    unsigned long long* full = mbar + 2 * R;   // STREAM: [2] a buffer's rows are there
     cg::cluster_group cl = cg::this_cluster();
     const int rank = (!ONE && C > 1) ? (int)cl.block_rank() : 0;
     const int tid = threadIdx.x, lane = tid & 31;
@@ -401,14 +478,35 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 ? 512 : 384), 1)
         if (grp[k] >= 0) first = grp[k];
     const int j = a.sys[first].sub;
     const int Pj = a.sub_P[j], Q = (Pj + 31) >> 5;
-    const FxSub f = a.fsub[j];
-    {   // rows of the separators this CTA holds (one contiguous piece), zero beyond them
+    FxSub f = a.fsub[(size_t)(STREAM ? a.fstep0 : 0) * (STREAM ? a.N : 0) + j];
+    const int have = max(0, min(T, S - rank * T)) * ROW;
+    // rows of the separators this CTA holds (one contiguous piece), zero beyond them.  STREAM:
+    // step t's rows and reduced system go to buffer t & 1 by one bulk copy each
+    auto fetch = [&](int t) {
+        const size_t st = a.fstep0 + (a.frev ? 1 - t : t - 1);
+        const unsigned dst = fx_saddr(fsm + (t & 1) * BUF), mb = fx_saddr(full + (t & 1));
+        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb),
+                     "r"(16u * (have + RD)) : "memory");
+        if (have)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(dst), "l"(a.rows + ((st * a.N + j) * S + rank * T) * ROW),
+                         "r"(16u * have), "r"(mb) : "memory");
+        if (RD)
+            asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
+                         ::"r"(dst + 16u * ROW * T), "l"(a.red + (st * a.N + j) * RD), "r"(16u * RD),
+                         "r"(mb) : "memory");
+    };
+    if (STREAM) {
+        for (int e = tid; e < 2 * BUF; e += blockDim.x) fsm[e] = make_int4(0, 0, 0, 0);
+        if (tid < 2) asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(fx_saddr(full + tid)) : "memory");
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+    } else {
         const int4* src = a.rows + ((size_t)j * S + rank * T) * ROW;
-        const int have = max(0, min(T, S - rank * T)) * ROW;
         for (int e = tid; e < ROW * T; e += blockDim.x) fsm[e] = e < have ? src[e] : make_int4(0, 0, 0, 0);
+        if (!ONE)
+            for (int e = tid; e < RD; e += blockDim.x) fsm[ROW * T + e] = a.red[(size_t)j * RD + e];
     }
     if (!ONE) {
-        for (int e = tid; e < 13 * 32; e += blockDim.x) srd[e] = a.red[(size_t)j * 13 * 32 + e];
         for (int e = tid; e < 4 * R * kFxSlots; e += blockDim.x) sA[e] = fx_zero();
         if (C > 1 && tid < 2 * R) {
             asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(fx_saddr(mbar + tid)) : "memory");
@@ -431,11 +529,17 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 ? 512 : 384), 1)
     const bool le = p == 0, re = p == Pj;
     // constants that round the shifts to nearest; ties (one in 2^k values) go up in odd steps
     // and down in even ones, so that they leave no mean behind
-    const int dd = f.sd - f.s2, ds2 = f.s2 - f.s;
-    const fx_int half_2 = f.s2 ? (fx_int)1 << (f.s2 - 1) : 0;
-    const fx_int half_z = ds2 ? (fx_int)1 << (ds2 - 1) : 0;
-    const fx_int half_d = dd ? (fx_int)1 << (dd - 1) : 0;
-    const int one_s = 1 << (29 - f.s);   // 2^-s as a high limb
+    int dd, ds2, one_s;   // one_s: 2^-s as a high limb
+    fx_int half_2, half_z, half_d;
+    auto scales = [&]() {
+        dd = f.sd - f.s2;
+        ds2 = f.s2 - f.s;
+        half_2 = f.s2 ? (fx_int)1 << (f.s2 - 1) : 0;
+        half_z = ds2 ? (fx_int)1 << (ds2 - 1) : 0;
+        half_d = dd ? (fx_int)1 << (dd - 1) : 0;
+        one_s = 1 << (29 - f.s);
+    };
+    scales();
     const int sc = act ? a.scale[sidx] : 0;
     FxC u[L], us = fx_zero(), usup = fx_zero();
     {
@@ -484,8 +588,25 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 ? 512 : 384), 1)
     // a warp without separators of its own takes no part (its system's barrier counts it)
     const int nsteps = (act && (C == 1 || q < nw)) ? sy.nt : 0;
     FxC fnext = (FLUX && fin && nsteps > 1) ? fin[1] : fx_zero();
+    // STREAM (one right-hand side per CTA): a CTA whose warps all sit out fetches nothing
+    if (STREAM && tid == 0 && nsteps > 1) fetch(2);
 #pragma unroll 1
     for (int t = 2; t <= nsteps; ++t) {
+        if (STREAM) {
+            f = a.fsub[(size_t)(a.fstep0 + (a.frev ? 1 - t : t - 1)) * a.N + j];
+            scales();
+            row = fsm + (t & 1) * BUF + t0 * ROW;
+            srd = fsm + (t & 1) * BUF + ROW * T;
+            if (ONE) {
+                __syncwarp();   // the other buffer has been read
+                if (tid == 0 && t < nsteps) fetch(t + 1);
+            }
+            late = !fx_wait(fx_saddr(full + (t & 1)), ((t - 2) >> 1) & 1);
+            if (__any_sync(0xffffffffu, late)) {
+                late = true;
+                break;
+            }
+        }
         const int tie = (t & 1) - 1;
         const fx_int r2 = half_2 + (f.s2 ? tie : 0), rz = half_z + (ds2 ? tie : 0);
         const fx_int rd = half_d + (dd ? tie : 0);
@@ -615,6 +736,8 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 ? 512 : 384), 1)
             } else {
                 __syncwarp();
             }
+            // every warp has pushed this step's rows, so it has read the last step's buffer
+            if (STREAM && tid == 0 && t < nsteps) fetch(t + 1);
             FxC x = fx_zero();
             if (lane <= Q) {
                 x = sA[(par * R + r) * kFxSlots + lane];
@@ -697,6 +820,10 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 ? 512 : 384), 1)
     }
     if (valid && ((mu >> 27) || (mv >> 27) || late)) a.bad[sidx] = 1;
     if (late) atomicOr(a.status, ST_TIMEOUT);
+    if (STREAM && late && tid == 0) {   // copies in flight, once more within the limit
+        fx_wait(fx_saddr(full), 0);
+        fx_wait(fx_saddr(full + 1), 0);
+    }
     if (valid && (sy.flags & (SYS_REC_LAST | SYS_WRITE_UT))) {
         const double s1 = fx_pow2(sh - sc);
         double2* last = (sy.flags & SYS_REC_LAST) && a.urec ? a.urec + sy.rec : nullptr;
@@ -717,8 +844,8 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 ? 512 : 384), 1)
 
 // Fluxes of steps 2..nt from the integer end traces (and the traces themselves for SYS_TRACE);
 // one CTA per system.  A trace keeps its absolute error, a few units, however small it is: an
-// impulse march with a trace that never reaches 2^40 units (2^-16 of the state), and an undriven
-// march from u0 with no trace that does, are flagged for FP64 instead.
+// impulse march with a trace that never reaches 2^40 units (2^-16 of the state), and any other
+// march with no trace (nor flux input) that does, are flagged for FP64 instead.
 __global__ void __launch_bounds__(128) k_fx_flux(const FxMarchArgs a, double2 two_sigma,
                                                  const double2* __restrict__ gin,
                                                  double2* __restrict__ gout,
@@ -729,11 +856,17 @@ __global__ void __launch_bounds__(128) k_fx_flux(const FxMarchArgs a, double2 tw
     if (a.bad[q]) return;
     const FxC* tr = reinterpret_cast<const FxC*>(a.trace) + (size_t)q * 2 * ntmax;
     const bool imp = sy.flags & (SYS_IMP_L | SYS_IMP_R);
-    if (sy.nt > 1 && a.scale[q] != 0 && !(a.fin && !a.tiny[q])) {
+    if (sy.nt > 1 && a.scale[q] != 0) {
         unsigned ml = 0, mr = 0;
         for (int t = 1 + threadIdx.x; t < sy.nt; t += blockDim.x) {
             if (tcf & 1) ml = fx_mag(ml, tr[t]);
             if (tcf & 2) mr = fx_mag(mr, tr[ntmax + t]);
+            if (a.driven) {   // the flux update's own input
+                const double big = scalbn(1.0, 40 - a.scale[q]);
+                for (int in : {sy.in_l, sy.in_r})
+                    if (in >= 0 && fmax(fabs(gin[(size_t)in + t].x), fabs(gin[(size_t)in + t].y)) >= big)
+                        ml |= 256u;
+            }
         }
         const bool bl = __syncthreads_or(ml >= 256u), br = __syncthreads_or(mr >= 256u);
         const bool hl = tcf & 1, hr = tcf & 2;
@@ -761,32 +894,32 @@ __global__ void __launch_bounds__(128) k_fx_flux(const FxMarchArgs a, double2 tw
 // ---------------------------------------------------------------------------
 // Launch shape: chunk length, CTAs per subdomain and threads per right-hand side.
 // ---------------------------------------------------------------------------
-static int fx_smem_bytes(int L, int T, int R, bool one) {
-    int b = 16 * (4 * L + 13) * T;
-    if (!one) b += 16 * 13 * 32 + 16 * 4 * R * kFxSlots + 16 * R;
+static int fx_smem_bytes(int L, int T, int R, bool one, bool stream) {
+    int b = 16 * ((4 * L + 13) * T + (one ? 0 : 13 * 32)) * (stream ? 2 : 1) + 16 * R + 16;
+    if (!one) b += 16 * 4 * R * kFxSlots;
     return b;
 }
 
 static int fx_tmax(int L) { return L == 16 ? 256 : (L == 4 ? 512 : 384); }
 
-bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out) {
+bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out, bool stream) {
     const int Ls[4] = {16, 12, 8, 4};
     double best = -1.0;
     for (int L : Ls) {
-        if (forceL && L != forceL) continue;
+        if ((forceL && L != forceL) || (stream && L > 8)) continue;
         const int S = (nmax - 1 + L) / (L + 1) + 1;   // separators
         if (S >= kTlMaxSep) continue;
         for (int C = 1; C <= 16; ++C) {
             const bool one = S <= 32;
             const int T = ((S + C - 1) / C + 31) / 32 * 32;
-            if ((one && C > 1) || R * T > fx_tmax(L) || (C > 1 && (C - 1) * T >= S)) continue;
-            const int smem = fx_smem_bytes(L, T, R, one);
+            if ((one && C > 1) || R * T > (stream ? std::min(384, fx_tmax(L)) : fx_tmax(L)) || (C > 1 && (C - 1) * T >= S)) continue;
+            const int smem = fx_smem_bytes(L, T, R, one, stream);
             if (smem > 220 * 1024) continue;
             // cycles a warp's step costs its SM sub-partition, and its own length (measured: 5000
             // and 9700 for a one-warp system with L = 12; 9800 for L = 4 over a cluster)
             const double iss = 320.0 * L + (one ? 1200.0 : 2600.0);
             const double lat = 620.0 * L + (one ? 2300.0 : 5800.0) + (C > 1 ? 1500.0 : 0.0);
-            const int regs = L == 16 ? 256 : (L == 4 ? 128 : 168);
+            const int regs = L == 16 ? 256 : (L == 4 && !stream ? 128 : 168);
             const int res = std::max(1, std::min(227 * 1024 / (smem + 1024), 65536 / (R * T * regs)));
             const double all = (double)ngroups * C;
             const double waves = std::ceil(all / ((double)nsm * res));
@@ -802,10 +935,10 @@ bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* ou
     return best >= 0.0;
 }
 
-template <int L, bool ONE, bool FLUX>
+template <int L, bool ONE, bool FLUX, bool STREAM>
 static int launch_fx_t(const FxMarchArgs& a, int ngroups, cudaStream_t s) {
-    const int smem = fx_smem_bytes(L, a.T, a.R, ONE);
-    auto kern = k_march_fx<L, ONE, FLUX>;
+    const int smem = fx_smem_bytes(L, a.T, a.R, ONE, STREAM);
+    auto kern = k_march_fx<L, ONE, FLUX, STREAM>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return -1;
     // several CTAs share an SM: all of its shared memory
@@ -833,13 +966,21 @@ static int launch_fx_t(const FxMarchArgs& a, int ngroups, cudaStream_t s) {
 
 template <int L>
 static int launch_fx_l(const FxMarchArgs& a, bool one, int ngroups, cudaStream_t s) {
-    if (a.fin) return one ? launch_fx_t<L, true, true>(a, ngroups, s) : launch_fx_t<L, false, true>(a, ngroups, s);
-    return one ? launch_fx_t<L, true, false>(a, ngroups, s) : launch_fx_t<L, false, false>(a, ngroups, s);
+    if constexpr (L <= 8) {   // per-step factors: latency bound, short chunks
+        if (a.stream) return one ? launch_fx_t<L, true, true, true>(a, ngroups, s)
+                                 : launch_fx_t<L, false, true, true>(a, ngroups, s);
+    }
+    if (a.stream) return -2;
+    if (a.fin) return one ? launch_fx_t<L, true, true, false>(a, ngroups, s)
+                          : launch_fx_t<L, false, true, false>(a, ngroups, s);
+    return one ? launch_fx_t<L, true, false, false>(a, ngroups, s)
+               : launch_fx_t<L, false, false, false>(a, ngroups, s);
 }
 
 int swr_launch_fx_start(const FactorSet& fs, FxMarchArgs a, int nsys, const double2* gin,
                         double2 inv_ik, cudaStream_t s) {
     a.fsub = fs.fx_sub;
+    a.stream = fs.nsteps > 1;
     k_fx_start<<<nsys, 256, 0, s>>>(a, gin, inv_ik);
     swr_count_launch(1);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
@@ -853,6 +994,8 @@ int swr_launch_march_fx(const FactorSet& fs, FxMarchArgs a, int ngroups, cudaStr
     a.fsub = fs.fx_sub;
     a.rows = fs.fx_rows;
     a.red = fs.fx_red;
+    a.stream = fs.nsteps > 1;
+    if (a.stream && (a.R != 1 || !a.fin)) return -2;
     const bool one = fs.P + 1 <= 32;
     if (one && (a.C != 1 || a.T != 32)) return -2;
     switch (fs.L) {
