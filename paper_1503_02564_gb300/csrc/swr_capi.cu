@@ -178,6 +178,12 @@ struct swr_plan_s {
     bool fac_stale[5] = {};              // fsL[] of another chunk length than the last build's
     int3* d_subsys = nullptr;            // per subdomain: its systems in the build list
     double2 *d_fxu = nullptr, *d_fxtrace = nullptr;
+    // S_0^2 ends: beta and c2 / (i kappa) 2^-fx_c2e as limbs, the history sums' scratch
+    int2* d_fxbeta = nullptr;
+    double2* d_fxhist = nullptr;
+    int4 fx_c2{};
+    int fx_c2e = 0;
+    double fx_hist = 0.0;                // |c2 / (i kappa)|
     unsigned long long* d_pit = nullptr;   // nonlinear marches: nodes x inner iterations
     double* d_scal = nullptr;      // [0] jump
     Workspace ws;
@@ -626,6 +632,9 @@ inline int march_kind(swr_plan_t p, bool zero_potential) {
     return MK_STATIC;
 }
 
+swr_status factor_for(swr_plan_t p, FactorSet& fs, int L, const double* V, double2* dg,
+                      double2* od);
+
 // The fixed-point form of a list's marches: step 1 in FP64 (it sets each system's scale), steps
 // 2..nt in fixed point, the fluxes from the end traces, and the flagged systems again in FP64.
 swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxList& fl,
@@ -633,6 +642,14 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
                         const double2* u0, long long work) {
     const int L = fl.sh.L;
     FactorSet& fs = zero_potential ? p->fs0L[lidx(L)] : p->fsL[lidx(L)];
+    // a chunk length that the build does not factor (and that a program may never march with):
+    // factored by the first march after the build
+    if (!zero_potential && p->d.vkind == SWR_V_STATIC && (fs.L != L || p->fac_stale[lidx(L)])) {
+        swr_status st = factor_for(p, fs, L, p->d_V, p->d_dg, p->d_od);
+        if (st) return st;
+        p->fac_stale[lidx(L)] = false;
+        p->fx_stale[lidx(L)] = true;
+    }
     if (fs.L != L) return SWR_ERR_STATE;
     const bool steps = fs.nsteps > 1;   // per-step factors
     const int kind = steps ? MK_TSTAT : MK_STATIC;
@@ -640,7 +657,7 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     const int pi = prof_begin(p, 0, work);
     int rc = 0;
     if (!zero_potential && !steps && p->fx_stale[lidx(L)]) {   // formed by the first march that needs it
-        rc = swr_launch_fx_prepare(fs, p->N, p->s);
+        rc = swr_launch_fx_prepare(fs, p->N, p->s, 0, 1, p->fx_hist);
         p->fx_stale[lidx(L)] = rc != 0;
     }
     SegArgs first, again;
@@ -672,6 +689,14 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     a.status = p->d_status;
     a.fin = fl.d_fin;
     a.driven = fl.driven && gin;
+    if (p->d_fxbeta) {
+        a.beta = p->d_fxbeta;
+        a.c2 = p->fx_c2;
+        a.c2e = p->fx_c2e;
+        a.u0 = u0;
+        a.htrace = p->d_fxhist;
+        a.two_c2 = make_double2(2.0 * p->c2.x, 2.0 * p->c2.y);
+    }
     a.N = p->N;
     a.fstep0 = first.fstep0;
     a.frev = first.frev;
@@ -1042,6 +1067,7 @@ swr_status fx_list(swr_plan_t p, swr_plan_s::FxList& fl, const MarchSys* sys, co
     if (!st && !p->d_fxu) {   // shared by the lists: the longest one is set up first
         st = dalloc(&p->d_fxu, (size_t)tot);
         if (!st) st = dalloc(&p->d_fxtrace, (size_t)nsys * 2 * p->nt);
+        if (!st && p->d.tc == SWR_TC_S02) st = dalloc(&p->d_fxhist, (size_t)nsys * 2 * p->nt);
     }
     if (st) return st;
     CK(cudaMemcpy(fl.d_grp, grp.data(), sizeof(int) * grp.size(), cudaMemcpyHostToDevice));
@@ -1686,6 +1712,7 @@ void swr_destroy(swr_plan_t p) {
         cudaFree(fl->d_fin);
     }
     cudaFree(p->d_subsys); cudaFree(p->d_fxu); cudaFree(p->d_fxtrace);
+    cudaFree(p->d_fxbeta); cudaFree(p->d_fxhist);
     cudaFree(p->d_W); cudaFree(p->d_spec); cudaFree(p->d_spec0); cudaFree(p->d_Gw);
     cudaFree(p->d_Pwin); cudaFree(p->d_hspec); cudaFree(p->d_hspec0);
     cudaFree(p->d_xspec);
@@ -1948,12 +1975,13 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
     for (const InstInfo& I : p->inst)
         for (int j = 0; j < I.N; ++j)
             crossed = crossed && (p->n[I.sub0 + j] - 1) * p->h <= I.nt * std::sqrt(d->dt);
-    const bool fx = fxR > 0 && d->tc == SWR_TC_ROBIN && !is_long && p->two_level && crossed &&
+    const bool fx_tc = d->tc == SWR_TC_ROBIN || (d->tc == SWR_TC_S02 && d->vkind == SWR_V_STATIC && p->nt <= 2048);
+    const bool fx = fxR > 0 && fx_tc && !is_long && p->two_level && crossed &&
                     p->nt >= 16 &&
                     swr_fx_shape(p->nmax, p->N, fxR, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fxs);
     // the marches of one system per subdomain (R g, final, the adjoint's d)
     FxShape fx1{};
-    const bool fx_one = d->vkind != SWR_V_NONLINEAR && d->tc == SWR_TC_ROBIN && !is_long &&
+    const bool fx_one = d->vkind != SWR_V_NONLINEAR && fx_tc && !is_long &&
                         p->two_level && p->nt >= 16 &&
                         (d->vkind != SWR_V_TIME || p->tune.tdep_precomp >= 0) &&
                         swr_fx_shape(p->nmax, p->N, 1, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fx1,
@@ -2043,6 +2071,24 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
         if (!st && cudaMemcpy(p->d_beta, beta.data(), sizeof(double) * (p->nt + 1),
                               cudaMemcpyHostToDevice) != cudaSuccess)
             st = SWR_ERR_CUDA;
+        if (!st && d->tc == SWR_TC_S02 && (fx || fx_one)) {
+            auto limbs = [](double c) {   // rint(c 2^61)
+                const long long C = (long long)std::llrint(std::ldexp(c, 61));
+                const int l = (int)(uint32_t)(uint64_t)C;
+                return make_int2((int)((C - l) >> 32), l);
+            };
+            std::vector<int2> bl(p->nt + 1);
+            for (int k = 0; k <= p->nt; ++k) bl[k] = limbs(beta[k]);
+            p->fx_hist = std::hypot(p->c2_ik.x, p->c2_ik.y);
+            p->fx_c2e = std::ilogb(p->fx_hist) + 1;
+            const int2 re = limbs(std::ldexp(p->c2_ik.x, -p->fx_c2e));
+            const int2 im = limbs(std::ldexp(p->c2_ik.y, -p->fx_c2e));
+            p->fx_c2 = make_int4(re.x, re.y, im.x, im.y);
+            st = dalloc(&p->d_fxbeta, bl.size());
+            if (!st && cudaMemcpy(p->d_fxbeta, bl.data(), sizeof(int2) * bl.size(),
+                                  cudaMemcpyHostToDevice) != cudaSuccess)
+                st = SWR_ERR_CUDA;
+        }
         if (!st)
             st = dalloc(&p->d_s02hist, (size_t)std::max(p->nsys_build, p->N) * 2 * (p->nt + 1));
     }
@@ -2161,9 +2207,9 @@ static swr_status build_body(swr_plan_t p, bool do_assemble) {
         // factorisations for the chunk lengths the marches of this plan will use
         const bool fx = p->fx_build.sys != nullptr;
         const int Lb = fx ? p->fx_build.sh.L : march_config(p, p->nsys_build).L;
-        const int La = p->fx_R.sys ? p->fx_R.sh.L : march_config(p, p->N).L;
+        const int La = p->fx_R.sys ? Lb : march_config(p, p->N).L;
         if ((st = factor_for(p, p->fsL[lidx(Lb)], Lb, p->d_V, p->d_dg, p->d_od))) return st;
-        if (fx) LK(swr_launch_fx_prepare(p->fsL[lidx(Lb)], p->N, s));
+        if (fx) LK(swr_launch_fx_prepare(p->fsL[lidx(Lb)], p->N, s, 0, 1, p->fx_hist));
         if (La != Lb && (st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od)))
             return st;
         CK(cudaMemsetAsync(p->d_iface, 0, sizeof(double2) * (nb + (size_t)p->ncols), s));
@@ -2192,7 +2238,7 @@ static swr_status build_body(swr_plan_t p, bool do_assemble) {
         const bool fx = p->fx_imp.sys != nullptr;
         const int L0 = fx ? p->fx_imp.sh.L : march_config(p, p->nsys_build - p->N).L;
         if ((st = factor_for(p, p->fs0L[lidx(L0)], L0, Vp, p->d_dg0, p->d_od0))) return st;
-        if (fx) LK(swr_launch_fx_prepare(p->fs0L[lidx(L0)], p->N, s));
+        if (fx) LK(swr_launch_fx_prepare(p->fs0L[lidx(L0)], p->N, s, 0, 1, p->fx_hist));
         CK(cudaMemsetAsync(p->d_iface0, 0, sizeof(double2) * (nb + (size_t)p->ncols), s));
         // impulse marches only (the first N systems of the build list are the d marches)
         st = run_march(p, true, p->d_sys_build + p->N, p->nsys_build - p->N, nullptr,
@@ -2286,7 +2332,7 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
     if (p->d.vkind == SWR_V_STATIC) {       // the chunk lengths this build factors
         for (auto& f : p->fac_stale) f = true;
         p->fac_stale[lidx(p->fx_build.sys ? p->fx_build.sh.L : march_config(p, p->nsys_build).L)] = false;
-        p->fac_stale[lidx(p->fx_R.sys ? p->fx_R.sh.L : march_config(p, p->N).L)] = false;
+        if (!p->fx_R.sys) p->fac_stale[lidx(march_config(p, p->N).L)] = false;
     }
     if (!p->built || !p->use_graph) {
         st = build_body(p, false);

@@ -294,6 +294,14 @@ struct FxMarchArgs {
     int driven;
     double2* uT;
     const int* sub_goff;
+    // S_0^2 ends (beta non-NULL): beta_0.. as limbs, c2 / (i kappa) 2^-c2e as limbs, the initial
+    // value, and the history sums b_n in units of 2^kFxHist, [nsys][2][nt]
+    const int2* beta;
+    int4 c2;
+    int c2e;
+    const double2* u0;
+    double2* htrace;
+    double2 two_c2;
     // per-step factors: subdomains N, the step-1 set and the direction of the walk
     int stream, N, fstep0, frev;
 };
@@ -361,8 +369,9 @@ int swr_march_tl_smem_bytes(int T);
 // threads per right-hand side for ngroups subdomains of at most nmax nodes (false: none).
 bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out,
                   bool stream = false);
-// (nb steps from t0 on, for per-step factors)
-int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0 = 0, int nb = 1);
+// (nb steps from t0 on, for per-step factors; hist: |c2 / (i kappa)| of S_0^2 ends, else 0)
+int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0 = 0, int nb = 1,
+                          double hist = 0.0);
 // Room for the fixed-point form of per-step factors (nsteps > 1), filled by
 // swr_launch_factor_steps: 0, -1 (no memory) or -2 (too many separators).
 size_t swr_fx_step_bytes(int N, int L, int P);

@@ -158,7 +158,8 @@ __global__ void __launch_bounds__(64) k_fx_bounds(
 
 // Scales of one subdomain from its maxima; eb, er, eC: exponents of 1/delta of the separators
 // and of the reduced system, and of its couplings.
-__device__ __forceinline__ FxSub fx_sub(const unsigned long long* mx, int& eb, int& er, int& eC) {
+__device__ __forceinline__ FxSub fx_sub(const unsigned long long* mx, double hist, int& eb, int& er,
+                                        int& eC) {
     auto get = [&](int k) { return __longlong_as_double((long long)mx[k]); };
     const double tiny = 1e-9;
     FxSub f = {};
@@ -174,7 +175,8 @@ __device__ __forceinline__ FxSub fx_sub(const unsigned long long* mx, int& eb, i
         }
         bad |= get(B_CO) > 1.1 || get(B_AX) > 2.6 || get(B_Y) > 4.0;
         // a separator's row: its stencil and a flux, the two chunks' parts
-        const double d0 = 2.0 * kFxF + get(B_D) + get(B_CZ);
+        // (and with S_0^2 ends a history term of a few times |c2 / (i kappa)| v, tested as it comes)
+        const double d0 = 2.0 * kFxF + get(B_D) + get(B_CZ) + 6.0 * hist;
         f.s = max(0, fx_clog2(fmax(get(B_Z), 1.0)) - 2);
         f.s2 = max(f.s, fx_clog2(fmax(d0, 1.0)) - 2);
         const double q = get(B_Q) * scalbn(1.0, f.s);
@@ -209,7 +211,7 @@ __global__ void __launch_bounds__(64) k_fx_convert(
     const double2* __restrict__ tl_pcr, const double2* __restrict__ tl_aux,
     const double2* __restrict__ tl_red, const unsigned long long* __restrict__ mx,
     FxSub* __restrict__ fsub, int4* __restrict__ rows, int4* __restrict__ red, long long fstride,
-    long long sstride, long long pstride) {
+    long long sstride, long long pstride, double hist) {
     const int j = blockIdx.y, S = P + 1, p = blockIdx.x * blockDim.x + threadIdx.x;
     const int Pj = sub_P[j], Q = (Pj + 31) / 32, N = gridDim.y;
     {   // batch entry z (per-step factors)
@@ -226,7 +228,7 @@ __global__ void __launch_bounds__(64) k_fx_convert(
         red += z * N * 13 * 32;
     }
     int eb, er, eC;
-    const FxSub f = fx_sub(mx + (size_t)j * B_N, eb, er, eC);
+    const FxSub f = fx_sub(mx + (size_t)j * B_N, hist, eb, er, eC);
     if (blockIdx.x == 0 && threadIdx.x == 0) fsub[j] = f;
     if (f.bad) return;
     const double2 zero = make_double2(0.0, 0.0);
@@ -319,7 +321,7 @@ int swr_fx_alloc_steps(FactorSet& fs, int N) {
     return 0;
 }
 
-int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0, int nb) {
+int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0, int nb, double hist) {
     const int S = fs.P + 1, one = S <= 32;
     if (fs.nsteps > 1 ? !fs.fx_steps : (!one && (!fs.tl_ok || fs.tl_rs != 32))) return -2;
     if (!fs.fx_sub && !fx_alloc(fs, N, 1, 1)) return -1;
@@ -336,7 +338,7 @@ int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0, int nb) 
                                      fs.fx_sub + (size_t)t0 * N,
                                      fs.fx_rows + (size_t)t0 * N * S * (4 * fs.L + 13),
                                      fs.fx_red + (size_t)t0 * N * 13 * 32, fs.fstride, fs.sstride,
-                                     fs.pstride);
+                                     fs.pstride, hist);
     swr_count_launch(2);
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
@@ -421,10 +423,11 @@ __global__ void __launch_bounds__(256) k_fx_start(const FxMarchArgs a, const dou
 // When a component passes the trigger the whole system is scaled down by 4: in the same step
 // if it is one warp, one step later otherwise, the word travelling in a spare bit of A.  End
 // traces (and through them the recorded states) carry the shift of their step.
-// FLUX: flux inputs (a.fin).
+// FLUX: flux inputs (a.fin).  HIST: S_0^2 ends.  STREAM: per-step factors.
 // Shared memory: a row of coefficients per chunk, once for all R (its odd length in 16-byte
 // units keeps a warp's reads free of bank conflicts), the reduced system, A and B.
 // ---------------------------------------------------------------------------
+constexpr int kFxHist = 1;    // history sums are kept in units of 2^kFxHist
 constexpr int kFxSlots = 34;   // A / B entries per right-hand side and parity
 
 __device__ __forceinline__ unsigned fx_saddr(const void* p) {
@@ -452,7 +455,42 @@ __device__ __forceinline__ bool fx_wait(unsigned mbar, unsigned parity) {
     return false;
 }
 
-template <int L, bool ONE, bool FLUX, bool STREAM>
+// S_0^2 history of one end, sum_{s<t} beta_{t-s} v_s, by one full warp in units of 2^kFxHist:
+// lanes strided over s, a fixed butterfly (every lane gets the sum).  v_0, v_1 in registers, v_s
+// at tr[s - 1] with its shift; the current shift is sh.
+__device__ __forceinline__ FxC fx_history(const int2* __restrict__ beta, FxC v0, FxC v1,
+                                          const FxC* tr, const int* tsh, int t, int sh, int lane) {
+    fx_int hr = 0, hi = 0, mr = 0, mi = 0;
+#pragma unroll 1
+    for (int s = lane; s < t; s += 32) {
+        const FxC x = s == 0 ? v0 : (s == 1 ? v1 : tr[s - 1]);
+        const int k = sh - (s < 2 ? 0 : tsh[s - 1]);
+        const FxS f = fx_split(FxC{x.r >> k, x.i >> k});
+        const int2 b = beta[t - s];
+        hr = fx_mw(f.rh, b.x, hr);
+        hi = fx_mw(f.ih, b.x, hi);
+        mr = fx_mw(f.rl, b.x, fx_mw(f.rh, b.y, mr));
+        mi = fx_mw(f.il, b.x, fx_mw(f.ih, b.y, mi));
+        hr += mr >> 32;
+        hi += mi >> 32;
+        mr &= 0xffffffffLL;
+        mi &= 0xffffffffLL;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        hr += __shfl_xor_sync(0xffffffffu, hr, off);
+        hi += __shfl_xor_sync(0xffffffffu, hi, off);
+        mr += __shfl_xor_sync(0xffffffffu, mr, off);
+        mi += __shfl_xor_sync(0xffffffffu, mi, off);
+    }
+    // (H 2^64 + M 2^32) / 2^61 / 2^kFxHist: sum |beta_s| < 36 for 2048 steps, so that |4 H| < 2^63
+    constexpr int e = 29 + kFxHist;
+    const fx_int half = (fx_int)1 << (e - 1);
+    const FxC a = {(hr << (3 - kFxHist)) + ((mr + half) >> e), (hi << (3 - kFxHist)) + ((mi + half) >> e)};
+    return a;
+}
+
+template <int L, bool ONE, bool FLUX, bool STREAM, bool HIST = false>
 __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384), 1)
     k_march_fx(const FxMarchArgs a) {
     constexpr int ROW = 4 * L + 13;
@@ -587,6 +625,20 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
     if (!ONE && C > 1) cl.sync(); else __syncthreads();
     // a warp without separators of its own takes no part (its system's barrier counts it)
     const int nsteps = (act && (C == 1 || q < nw)) ? sy.nt : 0;
+    // S_0^2: the warps that hold an end form its history; v_0 = u_0 and v_1 = (u_1 + u_0) / 2
+    const bool hist = HIST && act;
+    FxC v0 = fx_zero(), v1 = fx_zero();
+    if (hist && tr) {
+        const double s1 = fx_pow2(sc);
+        const double2 z = (sy.flags & SYS_ZERO_U0) ? make_double2(0.0, 0.0)
+                                                   : a.u0[a.sub_goff[j] + (le ? 0 : a.sub_n[j] - 1)];
+        if (fabs(z.x * s1) < 2.8e17 && fabs(z.y * s1) < 2.8e17) {   // 2^58
+            v0 = FxC{__double2ll_rn(z.x * s1), __double2ll_rn(z.y * s1)};
+            v1 = FxC{(us.r + v0.r) >> 1, (us.i + v0.i) >> 1};
+        } else {
+            mu = 0x80000000u;
+        }
+    }
     FxC fnext = (FLUX && fin && nsteps > 1) ? fin[1] : fx_zero();
     // STREAM (one right-hand side per CTA): a CTA whose warps all sit out fetches nothing
     if (STREAM && tid == 0 && nsteps > 1) fetch(2);
@@ -614,6 +666,22 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
         if (!ONE && C > 1 && t0 == 0)   // arm this CTA's barrier of the step
             asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
                              fx_saddr(mbar + par * R + r)), "r"(txb) : "memory");
+        FxC hb = fx_zero();   // this end's history sum
+        if (hist) {
+#pragma unroll 1
+            for (int side = 0; side < 2; ++side) {
+                if (!(tcf & (1 << side)) || q != (side ? Pj >> 5 : 0)) continue;   // uniform per warp
+                const int el = side ? Pj & 31 : 0;
+                const size_t o = ((size_t)sidx * 2 + side) * a.nt;
+                const FxC h = fx_history(a.beta, fx_from(v0, el), fx_from(v1, el),
+                                         reinterpret_cast<const FxC*>(a.trace) + o, a.tshift + o, t,
+                                         sh, lane);
+                if (lane == el && (side ? re : le)) {
+                    hb = h;
+                    reinterpret_cast<FxC*>(a.htrace)[o + t - 1] = h;
+                }
+            }
+        }
         // ---- forward: right-hand sides, elimination, left-end functional ------------------
         FxC uR = fx_down(us, 1);
         if (!ONE) {
@@ -659,6 +727,14 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
             d = fx_add(fx_shr_c(fo, f.s2, r2), dot);
             const FxC cl_ = fx_up(cr, 1);
             if (lane > 0 && !le) d = fx_add(d, cl_);
+            if (hist) {
+                const int kh = f.s2 - a.c2e - kFxHist;
+                FxAcc h = fx_acc_shr(kh);
+                fx_mac_full(h, fx_split(hb), a.c2);
+                d = fx_add(d, fx_res_shr(h, kh, mv));
+                mv |= fx_range<28>(0u, d) >> 2;
+                mv |= fx_range<28>(0u, hb) >> 2;
+            }
             if (!valid) d = fx_zero();
         }
         const FxC drow = d;
@@ -798,6 +874,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
             tr[t - 1] = v;
             tsh[t - 1] = sh;
         }
+        if (hist) __syncwarp();   // the next step's history reads them
         if (rec) record();
         const bool pass = __any_sync(0xffffffffu, ms >> (KT + 1));   // beyond the trigger
         if (pass) {
@@ -885,7 +962,13 @@ __global__ void __launch_bounds__(128) k_fx_flux(const FxMarchArgs a, double2 tw
         const int out = side ? sy.out_b : sy.out_a, in = side ? sy.in_r : sy.in_l;
         if (out >= 0 && gout) {
             const double2 g = (in >= 0 && gin) ? gin[(size_t)in + t] : make_double2(0.0, 0.0);
-            gout[(size_t)out + t] = csub(cmul(two_sigma, v), g);
+            double2 o2 = csub(cmul(two_sigma, v), g);
+            if (a.beta) {
+                const FxC h = reinterpret_cast<const FxC*>(a.htrace)[(size_t)q * 2 * ntmax + o];
+                const double s2 = s1 * (double)(1 << kFxHist);
+                o2 = cfma(a.two_c2, make_double2((double)h.r * s2, (double)h.i * s2), o2);
+            }
+            gout[(size_t)out + t] = o2;
         }
         if ((sy.flags & SYS_TRACE) && vtrace) vtrace[(size_t)q * 2 * ntmax + o] = v;
     }
@@ -935,10 +1018,10 @@ bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* ou
     return best >= 0.0;
 }
 
-template <int L, bool ONE, bool FLUX, bool STREAM>
+template <int L, bool ONE, bool FLUX, bool STREAM, bool HIST = false>
 static int launch_fx_t(const FxMarchArgs& a, int ngroups, cudaStream_t s) {
     const int smem = fx_smem_bytes(L, a.T, a.R, ONE, STREAM);
-    auto kern = k_march_fx<L, ONE, FLUX, STREAM>;
+    auto kern = k_march_fx<L, ONE, FLUX, STREAM, HIST>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return -1;
     // several CTAs share an SM: all of its shared memory
@@ -971,6 +1054,12 @@ static int launch_fx_l(const FxMarchArgs& a, bool one, int ngroups, cudaStream_t
                                  : launch_fx_t<L, false, true, true>(a, ngroups, s);
     }
     if (a.stream) return -2;
+    if (a.beta) {   // S_0^2 ends: instantiations of their own, so that Robin ones keep their registers
+        if (a.fin) return one ? launch_fx_t<L, true, true, false, true>(a, ngroups, s)
+                              : launch_fx_t<L, false, true, false, true>(a, ngroups, s);
+        return one ? launch_fx_t<L, true, false, false, true>(a, ngroups, s)
+                   : launch_fx_t<L, false, false, false, true>(a, ngroups, s);
+    }
     if (a.fin) return one ? launch_fx_t<L, true, true, false>(a, ngroups, s)
                           : launch_fx_t<L, false, true, false>(a, ngroups, s);
     return one ? launch_fx_t<L, true, false, false>(a, ngroups, s)
@@ -1066,22 +1155,27 @@ __device__ __forceinline__ double2 superpose_side_fx(const FxC* __restrict__ col
         __syncthreads();
         if (!in) continue;
         const int4* pc = reinterpret_cast<const int4*>(col + (size_t)k0 * stride);
-        for (int q = 0; q < kc; q += 4) {
-            FxAcc c = {hr, mr, hi, mi};
+        // eight states in flight per thread (loaded before any is used), folded every four
+        for (int q = 0; q < kc; q += 8) {
+            int4 v[8];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                if (q + e < kc) {
-                    const int4 v = __ldcs(pc + (size_t)(q + e) * stride);
+            for (int e = 0; e < 8; ++e)
+                v[e] = __ldcs(pc + (size_t)min(q + e, kc - 1) * stride);   // past the end: times zero
+#pragma unroll
+            for (int h = 0; h < 8; h += 4) {
+                FxAcc c = {hr, mr, hi, mi};
+#pragma unroll
+                for (int e = h; e < h + 4; ++e) {
                     FxC x;
-                    x.r = (fx_int)(((unsigned long long)(unsigned)v.y << 32) | (unsigned)v.x);
-                    x.i = (fx_int)(((unsigned long long)(unsigned)v.w << 32) | (unsigned)v.z);
+                    x.r = (fx_int)(((unsigned long long)(unsigned)v[e].y << 32) | (unsigned)v[e].x);
+                    x.i = (fx_int)(((unsigned long long)(unsigned)v[e].w << 32) | (unsigned)v[e].z);
                     fx_mac(c, fx_split(x), tile[q + e]);
                 }
+                hr = c.hr + (c.mr >> 32);
+                hi = c.hi + (c.mi >> 32);
+                mr = c.mr & 0xffffffffLL;
+                mi = c.mi & 0xffffffffLL;
             }
-            hr = c.hr + (c.mr >> 32);
-            hi = c.hi + (c.mi >> 32);
-            mr = c.mr & 0xffffffffLL;
-            mi = c.mi & 0xffffffffLL;
         }
     }
     // X C = H 2^64 + M 2^32, of scale 2^(sc + cb - eg)

@@ -33,10 +33,10 @@ def workload(sizes, nt, h=5e-4, p=None):
     return wl
 
 
-def march(wl, chunk, two_level, g):
+def march(wl, chunk, two_level, g, tc=0):
     from paper_1503_02564_gb300 import swr
     plan = swr.Plan(nx=wl.nx, a0=wl.a0, b0=wl.b0, nt=wl.nt, dt=wl.dt, nsub=wl.nsub, node_off=wl.off,
-                    p=wl.sigma, tuning={"chunk_L": chunk, "autotune": -1, "two_level": two_level})
+                    p=wl.sigma, tc=tc, tuning={"chunk_L": chunk, "autotune": -1, "two_level": two_level})
     plan.build_interface(torch.tensor(wl.V, device="cuda"), torch.tensor(wl.u0, device="cuda"))
     d = torch.zeros(plan.n_interface, dtype=torch.complex128, device="cuda")
     cols = torch.zeros(plan.n_cols, dtype=torch.complex128, device="cuda")
@@ -48,9 +48,9 @@ def march(wl, chunk, two_level, g):
     return d.cpu().numpy(), cols.cpu().numpy(), go.cpu().numpy()
 
 
-def problem(wl):
+def problem(wl, tc=0):
     return O.Problem(wl.a0, wl.b0, wl.nx, wl.dt, wl.nt, wl.off.astype(np.int64), wl.u0, wl.V,
-                     sigma=wl.sigma)
+                     tc=tc, sigma=wl.sigma)
 
 
 def check(wl, chunk, g=None, against_f64=True):
@@ -96,6 +96,27 @@ def test_driven_march_scales_its_state_down(chunk):
     wl = workload([400, 390, 1200], 64)
     g = W.random_interface(wl.nblk, wl.nt, 52) * (2.0 ** (40.0 * np.arange(wl.nt) / wl.nt))
     check(wl, chunk, g)
+
+
+@pytest.mark.parametrize("chunk,sizes", [
+    (4, [150, 40, 155]), (8, [31 * 9, 800, 290]), (12, [400, 415, 2000]), (16, [31 * 17, 520, 3001])])
+def test_s02_histories(chunk, sizes):
+    """S_0^2 ends: the end histories as integer sums, over more steps than lanes.  The columns of
+    an almost transparent condition are small differences of large terms (see test_gpu_long.py),
+    so they are measured against the extended-precision build, relative to the summands, and
+    the FP64 marches' distance to it is the yardstick for the plain errors."""
+    wl = workload(sizes, 90)
+    g = W.random_interface(wl.nblk, wl.nt, 51)
+    d1, c1, r1 = march(wl, chunk, 0, g, 1)
+    d0, c0, r0 = march(wl, chunk, -1, g, 1)
+    P = problem(wl, 1)
+    dx, cx, dm, cm = O.build_ext(P)
+    for a, b, x, mag in ((d1, d0, dx, dm), (c1, c0, cx, cm)):
+        e = np.linalg.norm((np.asarray(a, np.clongdouble).ravel() - np.ravel(x)).astype(np.complex128))
+        f = np.linalg.norm((np.asarray(b, np.clongdouble).ravel() - np.ravel(x)).astype(np.complex128))
+        assert e <= 1e-12 * np.linalg.norm(np.asarray(mag, np.float64).ravel())
+        assert e <= 3.0 * f + 1e-14 * np.linalg.norm(np.asarray(mag, np.float64).ravel())
+    assert rel(r1, r0) < 1e-11 and rel(r1, O.apply_R(P, g)) < TOL_MARCH
 
 
 @pytest.mark.parametrize("scale", [0.0, 1e-270, 1e-150, 1e150])
