@@ -168,11 +168,14 @@ struct swr_plan_s {
         int* d_shift = nullptr;          // [nsys][2][nt] its scalings-down, step by step
         double2* d_fin = nullptr;        // driven: [nsys][2][nt] converted inputs
         struct Launch {
-            int start, count, T;
+            int start, count, T, C;
         };
         std::vector<Launch> launches;
     };
     FxList fx_build, fx_imp, fx_d, fx_R, fx_final, fx_L;
+    std::vector<cudaStream_t> fx_side;   // launches of a list beside the first
+    cudaEvent_t fx_fork = nullptr;
+    std::vector<cudaEvent_t> fx_join;
     bool fx_tdep = false;                // V(t,x): the per-step factors have a fixed-point form
     bool fx_stale[5] = {};               // fsL[] whose fixed-point form is older than its factors
     bool fac_stale[5] = {};              // fsL[] of another chunk length than the last build's
@@ -672,7 +675,6 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
                         trace, u0, 1, first);
     FxMarchArgs a{};
     a.nt = p->nt;
-    a.C = fl.sh.C;
     a.R = fl.R;
     a.sys = fl.sys;
     a.sub_tc = p->d_tc;
@@ -701,10 +703,24 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     a.fstep0 = first.fstep0;
     a.frev = first.frev;
     if (!rc) rc = swr_launch_fx_start(fs, a, fl.nsys, gin, p->inv_ik, p->s);
-    for (const auto& g : fl.launches) {
+    // one launch per shape, side by side on the plan's side streams (forked from and joined to
+    // the plan's stream by events, in a capture as well)
+    const size_t side = p->fx_side.empty() ? 0 : fl.launches.size() - 1;
+    if (side && !rc && cudaEventRecord(p->fx_fork, p->s) != cudaSuccess) rc = -1;
+    for (size_t k = 0; k < fl.launches.size() && !rc; ++k) {
+        const auto& g = fl.launches[k];
         a.grp = fl.d_grp + (size_t)g.start * fl.R;
         a.T = g.T;
-        if (!rc) rc = swr_launch_march_fx(fs, a, g.count, p->s);
+        a.C = g.C;
+        cudaStream_t st = p->s;
+        if (side && k > 0) {
+            st = p->fx_side[k - 1];
+            if (cudaStreamWaitEvent(st, p->fx_fork, 0) != cudaSuccess) rc = -1;
+        }
+        if (!rc) rc = swr_launch_march_fx(fs, a, g.count, st);
+        if (!rc && st != p->s && (cudaEventRecord(p->fx_join[k - 1], st) != cudaSuccess ||
+                                  cudaStreamWaitEvent(p->s, p->fx_join[k - 1], 0) != cudaSuccess))
+            rc = -1;
     }
     if (!rc) rc = swr_launch_fx_flux(a, fl.nsys, p->two_sigma, gin, gout, trace, p->s);
     again.only = fl.d_bad;
@@ -1036,15 +1052,24 @@ swr_status fx_list(swr_plan_t p, swr_plan_s::FxList& fl, const MarchSys* sys, co
         one[q].rec = tot;
         tot += p->n[hs[q].sub];
     }
-    // one launch per number of warps a system takes (C = 1), the longest marches first
+    // one launch per shape: a cluster only where a system does not fit one CTA, as many warps as
+    // it takes; the longest marches first
+    std::vector<int> ctas(p->N, 1);
     for (int j = 0; j < p->N; ++j) {
         order[j] = j;
-        need[j] = sh.C > 1 ? sh.T : (chunks_for(p->n[j], sh.L) + 1 + 31) / 32 * 32;
+        const int S = chunks_for(p->n[j], sh.L) + 1;
+        need[j] = (S + 31) / 32 * 32;
+        if (sh.C > 1 && (!p->batched || need[j] > sh.C * sh.T / 2 ||
+                         !swr_fx_fits(sh.L, need[j], R, false, false))) {
+            ctas[j] = sh.C;
+            need[j] = sh.T;
+        }
     }
     std::vector<int> nts(p->N);
     for (const InstInfo& I : p->inst)
         for (int j = 0; j < I.N; ++j) nts[I.sub0 + j] = I.nt;
     std::stable_sort(order.begin(), order.end(), [&](int a, int b) {
+        if (ctas[a] != ctas[b]) return ctas[a] > ctas[b];
         return need[a] != need[b] ? need[a] > need[b] : nts[a] > nts[b];
     });
     std::vector<int> grp;
@@ -1052,8 +1077,8 @@ swr_status fx_list(swr_plan_t p, swr_plan_s::FxList& fl, const MarchSys* sys, co
         bool any = false;
         for (int k = 0; k < R; ++k) any |= of[(size_t)j * R + k] >= 0;
         if (!any) continue;
-        if (fl.launches.empty() || fl.launches.back().T != need[j])
-            fl.launches.push_back({(int)(grp.size() / R), 0, need[j]});
+        if (fl.launches.empty() || fl.launches.back().T != need[j] || fl.launches.back().C != ctas[j])
+            fl.launches.push_back({(int)(grp.size() / R), 0, need[j], ctas[j]});
         fl.launches.back().count += 1;
         for (int k = 0; k < R; ++k) grp.push_back(of[(size_t)j * R + k]);
     }
@@ -1075,6 +1100,15 @@ swr_status fx_list(swr_plan_t p, swr_plan_s::FxList& fl, const MarchSys* sys, co
     if (R == 3) {
         if ((st = dalloc(&p->d_subsys, (size_t)p->N))) return st;
         CK(cudaMemcpy(p->d_subsys, of.data(), sizeof(int3) * p->N, cudaMemcpyHostToDevice));
+    }
+    while (p->fx_side.size() + 1 < fl.launches.size()) {   // side streams of the later launches
+        cudaStream_t st = nullptr;
+        cudaEvent_t ev = nullptr;
+        if (!p->fx_fork) CK(cudaEventCreateWithFlags(&p->fx_fork, cudaEventDisableTiming));
+        CK(cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking));
+        p->fx_side.push_back(st);
+        CK(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        p->fx_join.push_back(ev);
     }
     fl.sys = sys;
     return SWR_OK;
@@ -1702,6 +1736,9 @@ void swr_destroy(swr_plan_t p) {
     cudaFree(p->d_sys_build); cudaFree(p->d_sys_R); cudaFree(p->d_sys_final); cudaFree(p->d_sys_L);
     cudaFree(p->d_status); cudaFree(p->d_scal); cudaFree(p->d_pit);
     cudaFree(p->d_urec); cudaFree(p->d_rec_base);
+    for (auto& st : p->fx_side) cudaStreamDestroy(st);
+    for (auto& e : p->fx_join) cudaEventDestroy(e);
+    if (p->fx_fork) cudaEventDestroy(p->fx_fork);
     for (auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final, &p->fx_L}) {
         cudaFree(fl->d_sys1);
         cudaFree(fl->d_grp);

@@ -98,11 +98,11 @@ __device__ __forceinline__ FxAcc fx_acc_shr(int k) {
     const fx_int half = (fx_int)1 << (28 + min(k, 3));
     return FxAcc{0, half, 0, half};
 }
-// (k < 0: m gets its top bit set where the result would not stay below 2^58)
-__device__ __forceinline__ FxC fx_res_shr(const FxAcc& a, int k, unsigned& m) {
+// (k < 0: m gets its top bit set where the result would not stay below 2^top)
+__device__ __forceinline__ FxC fx_res_shr(const FxAcc& a, int k, unsigned& m, int top = 58) {
     const int e = min(k, 3);
     if (k < 0) {
-        const int b = 55 + k;
+        const int b = top - 3 + k;
         const fx_int lim = (fx_int)1 << b;
         if ((unsigned long long)(a.hr + lim) >> (b + 1) || (unsigned long long)(a.hi + lim) >> (b + 1))
             m |= 0x80000000u;

@@ -369,6 +369,7 @@ int swr_march_tl_smem_bytes(int T);
 // threads per right-hand side for ngroups subdomains of at most nmax nodes (false: none).
 bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out,
                   bool stream = false);
+bool swr_fx_fits(int L, int T, int R, bool one, bool stream);   // T threads, R right-hand sides a CTA
 // (nb steps from t0 on, for per-step factors; hist: |c2 / (i kappa)| of S_0^2 ends, else 0)
 int swr_launch_fx_prepare(FactorSet& fs, int N, cudaStream_t s, int t0 = 0, int nb = 1,
                           double hist = 0.0);

@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                 const int kh = f.s2 - a.c2e - kFxHist;
                 FxAcc h = fx_acc_shr(kh);
                 fx_mac_full(h, fx_split(hb), a.c2);
-                d = fx_add(d, fx_res_shr(h, kh, mv));
+                d = fx_add(d, fx_res_shr(h, kh, mv, 60));
                 mv |= fx_range<28>(0u, d) >> 2;
                 mv |= fx_range<28>(0u, hb) >> 2;
             }
@@ -785,7 +785,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                 FxAcc c = fx_acc_shr(f.kc);
                 fx_mac(c, fx_split(y), srd[(up ? 12 : 11) * 32 + (qi & 31)]);
                 const FxC mine = (lane == 31 && !own_last) ? cr : drow;
-                FxC x = fx_add(fx_shr(mine, f.sr - f.s2), fx_res_shr(c, f.kc, mv));
+                FxC x = fx_add(fx_shr(mine, f.sr - f.s2), fx_res_shr(c, f.kc, mv, 60));
                 const bool isA = lane == 0 || own_last, isB = lane == 31 && !own_last;
                 if (isB && p >= Pj) x = fx_zero();
                 if (isA || isB) mv |= fx_range<28>(0u, x) >> 2;
@@ -983,7 +983,11 @@ static int fx_smem_bytes(int L, int T, int R, bool one, bool stream) {
     return b;
 }
 
-static int fx_tmax(int L) { return L == 16 ? 256 : (L == 4 ? 512 : 384); }
+// (threads: what the registers of an instantiation allow; shared memory: 220 KB)
+bool swr_fx_fits(int L, int T, int R, bool one, bool stream) {
+    const int tmax = L == 16 ? 256 : (L == 4 && !stream ? 512 : 384);
+    return R * T <= tmax && fx_smem_bytes(L, T, R, one, stream) <= 220 * 1024;
+}
 
 bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* out, bool stream) {
     const int Ls[4] = {16, 12, 8, 4};
@@ -995,9 +999,8 @@ bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* ou
         for (int C = 1; C <= 16; ++C) {
             const bool one = S <= 32;
             const int T = ((S + C - 1) / C + 31) / 32 * 32;
-            if ((one && C > 1) || R * T > (stream ? std::min(384, fx_tmax(L)) : fx_tmax(L)) || (C > 1 && (C - 1) * T >= S)) continue;
+            if ((one && C > 1) || !swr_fx_fits(L, T, R, one, stream) || (C > 1 && (C - 1) * T >= S)) continue;
             const int smem = fx_smem_bytes(L, T, R, one, stream);
-            if (smem > 220 * 1024) continue;
             // cycles a warp's step costs its SM sub-partition, and its own length (measured: 5000
             // and 9700 for a one-warp system with L = 12; 9800 for L = 4 over a cluster)
             const double iss = 320.0 * L + (one ? 1200.0 : 2600.0);
