@@ -57,8 +57,8 @@ __device__ __forceinline__ void cp_async_wait_all() {
 // P1 interpolant of W), scaled by 1/(i kappa).  dg[loff_j + i] is the diagonal,
 // od[loff_j + i] the coupling of local nodes i and i+1.
 // ---------------------------------------------------------------------------
-// The grid's constants come from the host: an FP64 division in every thread (seven of them)
-// made this kernel 11.8 us per 1000 nodes-steps of V(t,x) tables, against 3.2 us.
+// The grid's constants come from the host: with the FP64 divisions in every thread a batch of
+// 64 steps of a 60001-node V(t,x) table took 0.72 ms, without them 0.22 ms.
 struct AsmConsts {
     double h3, ih, h12, tdt, e_im;   // h/3, 1/h, h/12, 2/dt, (2/dt)(h/6)
 };

@@ -1,4 +1,5 @@
-// Constant-matrix subdomain marches in 64-bit fixed point (arithmetic: swr_fx.cuh).
+// Linear subdomain marches in 64-bit fixed point (arithmetic: swr_fx.cuh): constant matrices,
+// and V(t,x) with every step's factors streamed.
 //
 // The march and its partition into chunks and separators are those of swr_march.cu
 // (k_march_static, k_march_tl); the arithmetic is 5-6 times cheaper, which moves the limits:
@@ -36,6 +37,12 @@
 // trigger, non-finite data, factors outside the bounds, traces too small to keep enough bits,
 // see k_fx_flux) are marched again in FP64 by the kernels of swr_march.cu.  The first step,
 // which sets the scale, is always an FP64 one.
+//
+// Measured, build marches of 200001 nodes and 500 steps (zero flux, left and right impulse),
+// FP64 -> here: 500 subdomains 16.9 -> 4.5 ms, 256 19.4 -> 5.9, 64 19.3 -> 5.9, 16 20.1 -> 9.2
+// (bound by issue, about 240 instructions per node and step at 500; by a step's dependent
+// chain and its separators' exchange at 16).  V(t,x), 60001 nodes in 64 subdomains, 400 steps:
+// 4.7 -> 2.2 ms a march (one CTA of six warps per subdomain: the chain of a step, 5.6 us).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -1115,7 +1122,9 @@ int swr_launch_fx_flux(const FxMarchArgs& a, int nsys, double2 two_sigma, const 
 // nt > 512) the high sums stay below 2^62 over all steps; the middle sums are folded into
 // them every four steps.  A side marched in FP64 (flagged) is read as doubles in node order.
 //
-// FP64 form: 1.5 ms for 3.2 GB of states (200001 nodes, 500 steps), the FP64 pipe at 97 %.
+// Bound by memory: 0.80 ms for 3.2 GB of states (200001 nodes, 500 steps, 500 subdomains), with
+// eight states of a thread in flight (each used as it arrives: 1.2 ms).  The FP64 form, its pipe
+// at 97 %, takes 1.5 ms.
 // ---------------------------------------------------------------------------
 constexpr int kSupTile = 128;
 
