@@ -154,3 +154,42 @@ def test_gradient_follows_a_new_potential():
         out.append(grad.cpu().numpy())
         plan.destroy()
     assert rel(out[0], out[1]) < 1e-9
+
+
+@pytest.mark.parametrize("chunk,sizes", [
+    (12, [415, 31 * 13, 4121, 95 * 13, 2000, 64 * 13, 159 * 13]),   # 33, 32, 318, 96, 155, 65, 160 separators
+    (4, [2479, 310 * 5, 7, 127 * 5, 128 * 5]),                      # 497, 311, 3, 128, 129
+])
+def test_batch_with_every_size_of_cluster(chunk, sizes):
+    """Instances of uneven subdomains in one plan: one CTA, or a cluster of as many CTAs as the
+    subdomain takes, one launch per shape.  Each instance is marched to 1e-10 of the oracle, and
+    to 1e-12 of the FP64 marches of the same batch."""
+    from paper_1503_02564_gb300 import swr
+    wls = [workload(sizes, 130), workload(sizes[::-1], 100)]
+    insts = [dict(nx=w.nx, a0=w.a0, b0=w.b0, nt=w.nt, nsub=w.nsub, node_off=w.off) for w in wls]
+    gs = [W.random_interface(w.nblk, w.nt, 53 + k) for k, w in enumerate(wls)]
+    out = []
+    for two_level in (0, -1):
+        plan = swr.BatchPlan(insts, dt=wls[0].dt, p=wls[0].sigma, tc=0,
+                             tuning={"chunk_L": chunk, "autotune": -1, "two_level": two_level})
+        plan.build_interface(torch.tensor(np.concatenate([w.V for w in wls]), device="cuda"),
+                             torch.tensor(np.concatenate([w.u0 for w in wls]), device="cuda"))
+        d = torch.zeros(plan.n_interface, dtype=torch.complex128, device="cuda")
+        cols = torch.zeros(plan.n_cols, dtype=torch.complex128, device="cuda")
+        plan.get_interface(d, cols)
+        gi = torch.tensor(np.concatenate([g.ravel() for g in gs]), device="cuda")
+        go = torch.zeros_like(gi)
+        plan.apply_R(gi, go)
+        plan.destroy()
+        out.append([t.cpu().numpy() for t in (d, cols, go)])
+    for a, b in zip(*out):
+        assert rel(a, b) < 1e-12
+    d, cols, go = out[0]
+    kb = kc = 0
+    for w, g in zip(wls, gs):
+        P = problem(w)
+        assert rel(d[kb:kb + g.size], O.build_d(P)) < TOL_MARCH
+        assert rel(go[kb:kb + g.size], O.apply_R(P, g)) < TOL_MARCH
+        ref = O.build_columns(P)
+        assert rel(cols[kc:kc + np.size(ref)], ref) < TOL_MARCH
+        kb, kc = kb + g.size, kc + np.size(ref)
