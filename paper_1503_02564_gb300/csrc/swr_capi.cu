@@ -1056,7 +1056,7 @@ swr_status fx_list(swr_plan_t p, swr_plan_s::FxList& fl, const MarchSys* sys, co
     // in a batch, which fills the chip anyway, one CTA where half a cluster's threads are enough
     // (48 instances, 200 to 2000 nodes a subdomain: the build's marches in one launch of
     // clusters of five CTAs of 32 threads for each of three right-hand sides 26.2 ms; the whole
-    // solve with of five above 64 separators 31.0 ms, as here 28.3 ms)
+    // solve with clusters of five above 64 separators 31.0 ms, of the size each takes 28.3 ms)
     std::vector<int> ctas(p->N, 1);
     for (int j = 0; j < p->N; ++j) {
         order[j] = j;

@@ -25,6 +25,7 @@
 // for coefficients whose moduli sum to at most 2.6 (checked when they are converted).
 #pragma once
 
+#include <limits.h>
 #include <stdint.h>
 
 typedef long long fx_int;
@@ -72,12 +73,13 @@ __device__ __forceinline__ fx_int fx_mw(int a, int b, fx_int c) {
     asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(d) : "r"(a), "r"(b), "l"(c));
     return d;
 }
-// a += x c  (c: the limbs (re high, re low, im high, im low))
+// a += x c  (c: the limbs (re high, re low, im high, im low)).  The coefficient's limbs take the
+// minus sign: a low limb of x may be -2^31, whose negation wraps; fx_limbs makes no such one
 __device__ __forceinline__ void fx_mac(FxAcc& a, FxS x, int4 c) {
-    const int nih = -x.ih, nil = -x.il;
-    a.hr = fx_mw(nih, c.z, fx_mw(x.rh, c.x, a.hr));
+    const int nz = -c.z, nw = -c.w;
+    a.hr = fx_mw(x.ih, nz, fx_mw(x.rh, c.x, a.hr));
     a.mr = fx_mw(x.rl, c.x, fx_mw(x.rh, c.y, a.mr));
-    a.mr = fx_mw(nil, c.z, fx_mw(nih, c.w, a.mr));
+    a.mr = fx_mw(x.il, nz, fx_mw(x.ih, nw, a.mr));
     a.hi = fx_mw(x.ih, c.x, fx_mw(x.rh, c.z, a.hi));
     a.mi = fx_mw(x.rl, c.z, fx_mw(x.rh, c.w, a.mi));
     a.mi = fx_mw(x.il, c.x, fx_mw(x.ih, c.y, a.mi));
@@ -169,6 +171,7 @@ __device__ __forceinline__ int2 fx_limbs(double c) {
     const fx_int m = (b & 0xfffffffffffffLL) | (e > -1023 + 61 - 52 ? 0x10000000000000LL : 0);
     fx_int C = e >= 0 ? m << min(e, 10) : (e > -54 ? ((m >> (-e - 1)) + 1) >> 1 : 0);
     if (b < 0) C = -C;
+    C += (int)C == INT_MIN;   // its low limb has a negative (see fx_mac)
     const int l = (int)C;
     return make_int2((int)((C - l) >> 32), l);
 }
