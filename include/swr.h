@@ -156,7 +156,9 @@ typedef struct swr_tuning {
     int32_t two_level;          /* systems spread over a cluster: 0 (default) two-level  */
                                 /* separator solve (one cluster barrier per step) when   */
                                 /* a system has <= 993 separators (the nonlinear         */
-                                /* gradient's monodomain: <= 8161); -1 cluster-wide PCR  */
+                                /* gradient's monodomain: <= 8161); -1 cluster-wide PCR, */
+                                /* and the linear marches in FP64 instead of 64-bit      */
+                                /* fixed point (Robin, Neumann and S_0^2 ends, nt >= 16) */
     int32_t debug;              /* 1: failing CUDA calls (2: also the launch-shape      */
                                 /* probes) reported on stderr; 0 (default) silent        */
     int32_t history_fft;        /* causal substitution (CAUSAL preconditioner, direct   */
