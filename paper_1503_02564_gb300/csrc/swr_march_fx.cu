@@ -1018,7 +1018,12 @@ bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* ou
             const double waves = std::ceil(all / ((double)nsm * res));
             const double ctas = std::min((double)res, std::ceil(all / nsm));
             const double warps = ctas * R * (T / 32) / 4.0;   // per SM sub-partition
-            const double step = waves * std::max(lat, std::max(warps, 1.0) * iss);
+            double step = waves * std::max(lat, std::max(warps, 1.0) * iss);
+            // four-node chunks only where they are clearly faster: the factors of more separators
+            // carry more rounding error (R g of 200001 nodes, 256 subdomains, 500 steps, against
+            // extended precision: 5.8e-12 with 4 nodes, 3.3e-12 with 8, 2.7e-12 with 12, in FP64
+            // the same) and the march gains nothing (that R g: 3.65 ms with 4, 3.54 ms with 8)
+            if (L == 4 && !stream) step *= 1.25;
             if (best < 0.0 || step < best) {
                 best = step;
                 *out = FxShape{L, C, T};
