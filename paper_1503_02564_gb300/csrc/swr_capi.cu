@@ -395,6 +395,7 @@ struct SegArgs {
     const double2* vfwd = nullptr;
     double *gint = nullptr, *gl = nullptr, *gr = nullptr;
     double2* urec = nullptr;        // recorded states (NULL: the plan's)
+    bool record = true;             // false: record no states
     const int* only = nullptr;      // march only the flagged systems
     int tstride = 0;                // entries per trace (0: the launch's own step count)
 };
@@ -573,7 +574,8 @@ int launch_cfg(swr_plan_t p, const MarchCfg& cfg, int kind, bool zero_potential,
     a.gout = gout;
     a.uT = uT;
     a.trace = trace;
-    a.urec = seg.urec ? seg.urec : ((!zero_potential && p->superpose) ? p->d_urec : nullptr);
+    a.urec = seg.urec ? seg.urec
+                      : ((!zero_potential && p->superpose && seg.record) ? p->d_urec : nullptr);
     a.only = seg.only;
     a.tstride = seg.tstride;
     a.two_sigma = p->two_sigma;
@@ -642,7 +644,7 @@ swr_status factor_for(swr_plan_t p, FactorSet& fs, int L, const double* V, doubl
 // 2..nt in fixed point, the fluxes from the end traces, and the flagged systems again in FP64.
 swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxList& fl,
                         const double2* gin, double2* gout, double2* uT, double2* trace,
-                        const double2* u0, long long work) {
+                        const double2* u0, long long work, bool record) {
     const int L = fl.sh.L;
     FactorSet& fs = zero_potential ? p->fs0L[lidx(L)] : p->fsL[lidx(L)];
     // a chunk length that the build does not factor (and that a program may never march with):
@@ -682,7 +684,7 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     a.sub_goff = p->d_goff;
     a.soff = fl.d_soff;
     a.u1 = p->d_fxu;
-    a.urec = (!zero_potential && p->superpose) ? p->d_urec : nullptr;
+    a.urec = (!zero_potential && p->superpose && record) ? p->d_urec : nullptr;
     a.uT = uT;
     a.trace = p->d_fxtrace;
     a.scale = fl.d_scale;
@@ -724,6 +726,7 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     }
     if (!rc) rc = swr_launch_fx_flux(a, fl.nsys, p->two_sigma, gin, gout, trace, p->s);
     again.only = fl.d_bad;
+    again.record = record;
     if (!rc)
         rc = launch_cfg(p, cfg, kind, zero_potential, fl.sys, fl.nsys, gin, gout, uT, trace, u0,
                         p->nt, again);
@@ -731,18 +734,22 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     return rc ? launch_fail("march (fixed point)", __LINE__) : SWR_OK;
 }
 
-// vrec (nonlinear marches only): also record v_n of every step, rows of nx values
+// vrec (nonlinear marches only): also record v_n of every step, rows of nx values; record = false:
+// the states that the list's flags name are not recorded (the adjoint marches the build's
+// zero-flux systems from another state, and u(T) is still superposed from the build's)
 swr_status run_march(swr_plan_t p, bool zero_potential, const MarchSys* d_sys, int nsys,
                      const double2* gin, double2* gout, double2* uT, double2* trace,
-                     const double2* u0, long long work, double2* vrec = nullptr) {
+                     const double2* u0, long long work, double2* vrec = nullptr,
+                     bool record = true) {
     const int kind = march_kind(p, zero_potential);
     for (const auto* fl : {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final, &p->fx_L})
         if ((kind == MK_STATIC || (kind == MK_TSTAT && p->fx_tdep)) && fl->sys && fl->sys == d_sys &&
             fl->nsys == nsys && !vrec)
-            return run_march_fx(p, zero_potential, *fl, gin, gout, uT, trace, u0, work);
+            return run_march_fx(p, zero_potential, *fl, gin, gout, uT, trace, u0, work, record);
     const MarchCfg cfg = march_config(p, nsys, kind);
     const int pi = prof_begin(p, kind == MK_NL ? 3 : 0, work);
     SegArgs sa;
+    sa.record = record;
     if (vrec) {
         if (kind != MK_NL) return SWR_ERR_UNSUPPORTED;
         sa.mode = 1;
@@ -2913,7 +2920,7 @@ swr_status swr_adjoint(swr_plan_t p, const double* ubar_, double* dJdV_, int32_t
     LK(swr_launch_adj_seed(reinterpret_cast<const double2*>(ubar_), 0.5 * p->d.dt, nx, p->d_ya, s));
     CK(cudaMemsetAsync(p->d_dy, 0, sizeof(double2) * nb, s));
     if ((st = run_march(p, false, p->d_sys_build, N, nullptr, p->d_dy, nullptr, nullptr, p->d_ya,
-                        p->work_R)))
+                        p->work_R, nullptr, false)))
         return st;
     double dn = 0.0, dny = 0.0;
     if ((st = norm2(p, p->d_iface, (long long)nb, &dn)) || (st = norm2(p, p->d_dy, (long long)nb, &dny)))
