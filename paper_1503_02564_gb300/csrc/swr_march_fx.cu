@@ -624,6 +624,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
     }
     unsigned mu = 0, mv = 0;
     bool grown = false, late = false;
+    int tlate = 0;   // STREAM: the step whose wait ran out
     const int nw = Pj / 32 + 1;            // warps of the system that hold separators
     const int ncta = Pj / T + 1;           // CTAs of the cluster that do
     // bytes a step pushes to each of them: A[0..Q], and B of every warp whose lane 31 is not
@@ -661,8 +662,10 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                 if (tid == 0 && t < nsteps) fetch(t + 1);
             }
             late = !fx_wait(fx_saddr(full + (t & 1)), ((t - 2) >> 1) & 1);
-            if (__any_sync(0xffffffffu, late)) {
-                late = true;
+            late = __any_sync(0xffffffffu, late);
+            // a system of several warps in one CTA gives up together, at the step's barrier
+            if (late && (ONE || C > 1 || T == 32)) {
+                tlate = t;
                 break;
             }
         }
@@ -814,6 +817,19 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                     fx_wait(fx_saddr(mbar + par * R + r), ((t - 2) >> 1) & 1);
                     break;
                 }
+            } else if (STREAM && T > 32) {
+                // with the warps' late flags: one that left its loop alone would leave the others
+                // at this barrier without a limit (the rows it worked on are not there, so what
+                // it put into A and B is never used)
+                int any;
+                asm volatile("{\n\t.reg .pred q;\n\tsetp.ne.s32 q, %3, 0;\n\t"
+                             "barrier.cta.red.or.pred q, %1, %2, q;\n\tselp.s32 %0, 1, 0, q;\n\t}"
+                             : "=r"(any) : "r"(r + 1), "r"(T), "r"((int)late) : "memory");
+                if (any) {
+                    late = true;
+                    tlate = t;
+                    break;
+                }
             } else if (T > 32) {
                 asm volatile("bar.sync %0, %1;" ::"r"(r + 1), "r"(T) : "memory");
             } else {
@@ -904,9 +920,9 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
     }
     if (valid && ((mu >> 27) || (mv >> 27) || late)) a.bad[sidx] = 1;
     if (late) atomicOr(a.status, ST_TIMEOUT);
-    if (STREAM && late && tid == 0) {   // copies in flight, once more within the limit
-        fx_wait(fx_saddr(full), 0);
-        fx_wait(fx_saddr(full + 1), 0);
+    if (STREAM && tlate && tid == 0) {   // copies in flight, once more within the limit
+        fx_wait(fx_saddr(full + (tlate & 1)), ((tlate - 2) >> 1) & 1);
+        if (ONE && tlate < nsteps) fx_wait(fx_saddr(full + ((tlate + 1) & 1)), ((tlate - 1) >> 1) & 1);
     }
     if (valid && (sy.flags & (SYS_REC_LAST | SYS_WRITE_UT))) {
         const double s1 = fx_pow2(sh - sc);
