@@ -176,6 +176,7 @@ struct swr_plan_s {
     std::vector<cudaStream_t> fx_side;   // launches of a list beside the first
     cudaEvent_t fx_fork = nullptr;
     std::vector<cudaEvent_t> fx_join;
+    bool fx_full = false;                // whole products (see plan_create)
     bool fx_tdep = false;                // V(t,x): the per-step factors have a fixed-point form
     bool fx_stale[5] = {};               // fsL[] whose fixed-point form is older than its factors
     bool fac_stale[5] = {};              // fsL[] of another chunk length than the last build's
@@ -693,6 +694,7 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
     a.status = p->d_status;
     a.fin = fl.d_fin;
     a.driven = fl.driven && gin;
+    a.full = p->fx_full;
     if (p->d_fxbeta) {
         a.beta = p->d_fxbeta;
         a.c2 = p->fx_c2;
@@ -2022,7 +2024,19 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
     for (const InstInfo& I : p->inst)
         for (int j = 0; j < I.N; ++j)
             crossed = crossed && (p->n[I.sub0 + j] - 1) * p->h <= I.nt * std::sqrt(d->dt);
-    const bool fx_tc = d->tc == SWR_TC_ROBIN || (d->tc == SWR_TC_S02 && d->vkind == SWR_V_STATIC && p->nt <= 2048);
+    // Rounding of the factors, the same here and in FP64, makes an error of about 1e-16 dt / h^2 per
+    // step.  On coarse grids it no longer covers the march's own rounding.  Errors of the build's
+    // columns against extended precision, FP64, here, and here with the products of the low limbs
+    // (150 steps of 1e-3): dt/h^2 = 62 1.3e-14 all three; 16 6.4e-15, 6.6e-15, 6.5e-15; 4 2.8e-15,
+    // 3.4e-15, 3.2e-15; 1.7 (200 steps) 1.4e-15, 2.9e-15, 1.4e-15.  Whole products cost 7 to 20 % of
+    // a solve, so they are taken below 32 only.  S_0^2 ends always take them (with them the errors
+    // at dt/h^2 = 4000 are the FP64 ones, without them up to twice those in single blocks of
+    // R g); on coarse grids, where they still leave up to 1.4 times the FP64 error (8.5e-15
+    // against 6.3e-15 at 1.6), such plans march in FP64.
+    const bool coarse = d->dt < 32.0 * p->h * p->h;
+    p->fx_full = coarse;
+    const bool fx_tc = d->tc == SWR_TC_ROBIN ||
+                       (d->tc == SWR_TC_S02 && d->vkind == SWR_V_STATIC && p->nt <= 2048 && !coarse);
     const bool fx = fxR > 0 && fx_tc && !is_long && p->two_level && crossed &&
                     p->nt >= 16 &&
                     swr_fx_shape(p->nmax, p->N, fxR, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fxs);
@@ -2521,7 +2535,8 @@ swr_status swr_solve(swr_plan_t p, double* g_, int32_t g_is_initial, double* uT_
             LK(swr_launch_superpose_fx(p->fsL[lidx(p->fx_build.sh.L)], p->d_urec, p->d_rec_base,
                                        p->d_sys_final, p->d_subsys, p->N, p->d_n, p->d_goff,
                                        p->d_tc, p->fx_build.d_scale, p->fx_build.d_shift, p->nt,
-                                       p->fx_build.d_bad, g, uT, s));
+                                       p->fx_build.d_bad, g, uT,
+                                       p->fx_full || p->d.tc == SWR_TC_S02, s));
         else if (uT)
             LK(swr_launch_superpose(p->d_urec, p->d_rec_base, p->d_sys_final, p->N, p->d_n,
                                     p->d_goff, p->d_tc, p->nmax, g, uT, s));

@@ -92,6 +92,12 @@ __device__ __forceinline__ void fx_mac_full(FxAcc& a, FxS x, int4 c) {
     a.mr += (fx_int)__mulhi(x.rl, c.y) - __mulhi(x.il, c.w);
     a.mi += (fx_int)__mulhi(x.rl, c.w) + __mulhi(x.il, c.y);
 }
+// fx_mac, or fx_mac_full where a march takes all its products whole (FULL, see swr_march_fx.cu)
+template <bool FULL>
+__device__ __forceinline__ void fx_mul(FxAcc& a, FxS x, int4 c) {
+    if constexpr (FULL) fx_mac_full(a, x, c);
+    else fx_mac(a, x, c);
+}
 __device__ __forceinline__ FxC fx_res(const FxAcc& a) {
     return FxC{8 * a.hr + (a.mr >> 29), 8 * a.hi + (a.mi >> 29)};
 }

@@ -302,6 +302,7 @@ struct FxMarchArgs {
     const double2* u0;
     double2* htrace;
     double2 two_c2;
+    int full;             // all products whole (coarse grids; S_0^2 ends always)
     // per-step factors: subdomains N, the step-1 set and the direction of the walk
     int stream, N, fstep0, frev;
 };
@@ -386,7 +387,7 @@ int swr_launch_superpose_fx(const FactorSet& fs, const double2* urec, const long
                             const MarchSys* sys, const int3* subsys, int N, const int* sub_n,
                             const int* sub_goff, const int* sub_tc, const int* scale,
                             const int* shift, int ntmax, const int* bad, const double2* g,
-                            double2* uT, cudaStream_t s);
+                            double2* uT, int full, cudaStream_t s);
 
 // Interface algebra launchers (swr_krylov.cu)
 int swr_launch_toeplitz(int N, int nt, const double2* cols, const double2* x, const double2* add,

@@ -430,7 +430,8 @@ __global__ void __launch_bounds__(256) k_fx_start(const FxMarchArgs a, const dou
 // When a component passes the trigger the whole system is scaled down by 4: in the same step
 // if it is one warp, one step later otherwise, the word travelling in a spare bit of A.  End
 // traces (and through them the recorded states) carry the shift of their step.
-// FLUX: flux inputs (a.fin).  HIST: S_0^2 ends.  STREAM: per-step factors.
+// FLUX: flux inputs (a.fin).  HIST: S_0^2 ends.  STREAM: per-step factors.  FULL: the products of
+// the low limbs too, everywhere (coarse grids and S_0^2 ends, see plan_create).
 // Shared memory: a row of coefficients per chunk, once for all R (its odd length in 16-byte
 // units keeps a warp's reads free of bank conflicts), the reduced system, A and B.
 // ---------------------------------------------------------------------------
@@ -472,12 +473,15 @@ __device__ __forceinline__ FxC fx_history(const int2* __restrict__ beta, FxC v0,
     for (int s = lane; s < t; s += 32) {
         const FxC x = s == 0 ? v0 : (s == 1 ? v1 : tr[s - 1]);
         const int k = sh - (s < 2 ? 0 : tsh[s - 1]);
-        const FxS f = fx_split(FxC{x.r >> k, x.i >> k});
+        const fx_int half = ((fx_int)1 << k) >> 1;
+        const FxS f = fx_split(FxC{(x.r + half) >> k, (x.i + half) >> k});
         const int2 b = beta[t - s];
         hr = fx_mw(f.rh, b.x, hr);
         hi = fx_mw(f.ih, b.x, hi);
         mr = fx_mw(f.rl, b.x, fx_mw(f.rh, b.y, mr));
         mi = fx_mw(f.il, b.x, fx_mw(f.ih, b.y, mi));
+        mr += __mulhi(f.rl, b.y);
+        mi += __mulhi(f.il, b.y);
         hr += mr >> 32;
         hi += mi >> 32;
         mr &= 0xffffffffLL;
@@ -497,7 +501,7 @@ __device__ __forceinline__ FxC fx_history(const int2* __restrict__ beta, FxC v0,
     return a;
 }
 
-template <int L, bool ONE, bool FLUX, bool STREAM, bool HIST = false>
+template <int L, bool ONE, bool FLUX, bool STREAM, bool HIST, bool FULL>
 __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384), 1)
     k_march_fx(const FxMarchArgs a) {
     constexpr int ROW = 4 * L + 13;
@@ -707,9 +711,9 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
             const FxS fs = fx_split(fi);
             FxAcc c = fx_acc();
             fx_mac_pow2(c, fs, one_s);
-            if (i) fx_mac(c, fx_split(z[i > 0 ? i - 1 : 0]), row[4 * (i > 0 ? i - 1 : 0) + 1]);
+            if (i) fx_mul<FULL>(c, fx_split(z[i > 0 ? i - 1 : 0]), row[4 * (i > 0 ? i - 1 : 0) + 1]);
             z[i] = fx_res(c);
-            fx_mac(da, fs, row[4 * i + 2]);
+            fx_mul<FULL>(da, fs, row[4 * i + 2]);
             if (i & 1) {   // |f| < 2^61: at most four products between foldings
                 dot = fx_add(dot, fx_res(da));
                 da = fx_acc();
@@ -726,7 +730,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
         FxC cr, d;   // cr: this chunk's part of its right separator's row
         {
             FxAcc c = fx_acc();
-            fx_mac(c, fx_split(z[L - 1]), row[4 * (L - 1) + 1]);
+            fx_mul<FULL>(c, fx_split(z[L - 1]), row[4 * (L - 1) + 1]);
             cr = fx_add(fx_shr_c(u[L - 1], f.s2, r2), fx_shr_c(fx_res(c), ds2, rz));
             FxC fo = (le || re) ? FxC{2 * us.r, 2 * us.i} : FxC{4 * us.r, 4 * us.i};
             if (!re) fo = fx_add(fo, uf);
@@ -765,8 +769,8 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
             dp.ih = __shfl_down_sync(0xffffffffu, ds.ih, st);
             dp.il = __shfl_down_sync(0xffffffffu, ds.il, st);
             FxAcc c = fx_acc();
-            fx_mac(c, dm, row[4 * L + 2 * k]);
-            fx_mac(c, dp, row[4 * L + 2 * k + 1]);
+            fx_mul<FULL>(c, dm, row[4 * L + 2 * k]);
+            fx_mul<FULL>(c, dp, row[4 * L + 2 * k + 1]);
             d = fx_add(d, fx_res(c));
             mv |= fx_range<28>(0u, d) >> 2;   // to the bit of fx_range<26>
         }
@@ -793,7 +797,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                 FxC y = up ? yf : yl;
                 if (m == 0 || (lane == 0 && re)) y = fx_zero();
                 FxAcc c = fx_acc_shr(f.kc);
-                fx_mac(c, fx_split(y), srd[(up ? 12 : 11) * 32 + (qi & 31)]);
+                fx_mul<FULL>(c, fx_split(y), srd[(up ? 12 : 11) * 32 + (qi & 31)]);
                 const FxC mine = (lane == 31 && !own_last) ? cr : drow;
                 FxC x = fx_add(fx_shr(mine, f.sr - f.s2), fx_res_shr(c, f.kc, mv, 60));
                 const bool isA = lane == 0 || own_last, isB = lane == 31 && !own_last;
@@ -852,8 +856,8 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                 const FxC xm = fx_up(x, st), xp = fx_down(x, st);
                 FxAcc c = fx_acc();
                 mv |= fx_range<28>(0u, x) >> 2;
-                fx_mac(c, fx_split(xm), srd[(2 * k) * 32 + lane]);
-                fx_mac(c, fx_split(xp), srd[(2 * k + 1) * 32 + lane]);
+                fx_mul<FULL>(c, fx_split(xm), srd[(2 * k) * 32 + lane]);
+                fx_mul<FULL>(c, fx_split(xp), srd[(2 * k + 1) * 32 + lane]);
                 x = fx_add(x, fx_res(c));
             }
             mv |= fx_range<28>(0u, x) >> 2;
@@ -882,9 +886,9 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
 #pragma unroll
             for (int i = L - 1; i >= 0; --i) {
                 FxAcc c = fx_acc();
-                fx_mac(c, fx_split(z[i]), row[4 * i]);
-                fx_mac(c, vl, row[4 * i + 3]);
-                fx_mac(c, xs, row[4 * i + 1]);
+                fx_mul<FULL>(c, fx_split(z[i]), row[4 * i]);
+                fx_mul<FULL>(c, vl, row[4 * i + 3]);
+                fx_mul<FULL>(c, xs, row[4 * i + 1]);
                 const FxC x = fx_res(c);
                 xs = fx_split(x);
                 u[i] = fx_twice_less(x, u[i]);
@@ -1049,10 +1053,10 @@ bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* ou
     return best >= 0.0;
 }
 
-template <int L, bool ONE, bool FLUX, bool STREAM, bool HIST = false>
+template <int L, bool ONE, bool FLUX, bool STREAM, bool HIST, bool FULL>
 static int launch_fx_t(const FxMarchArgs& a, int ngroups, cudaStream_t s) {
     const int smem = fx_smem_bytes(L, a.T, a.R, ONE, STREAM);
-    auto kern = k_march_fx<L, ONE, FLUX, STREAM, HIST>;
+    auto kern = k_march_fx<L, ONE, FLUX, STREAM, HIST, FULL>;
     if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem) != cudaSuccess)
         return -1;
     // several CTAs share an SM: all of its shared memory
@@ -1078,23 +1082,27 @@ static int launch_fx_t(const FxMarchArgs& a, int ngroups, cudaStream_t s) {
     return cudaLaunchKernelEx(&cfg, kern, a) == cudaSuccess ? 0 : -1;
 }
 
+template <int L, bool FLUX, bool STREAM, bool HIST>
+static int launch_fx_f(const FxMarchArgs& a, bool one, bool full, int ngroups, cudaStream_t s) {
+    if (full) return one ? launch_fx_t<L, true, FLUX, STREAM, HIST, true>(a, ngroups, s)
+                         : launch_fx_t<L, false, FLUX, STREAM, HIST, true>(a, ngroups, s);
+    if constexpr (HIST) return -2;
+    else return one ? launch_fx_t<L, true, FLUX, STREAM, HIST, false>(a, ngroups, s)
+                    : launch_fx_t<L, false, FLUX, STREAM, HIST, false>(a, ngroups, s);
+}
+
 template <int L>
 static int launch_fx_l(const FxMarchArgs& a, bool one, int ngroups, cudaStream_t s) {
+    const bool full = a.full;
     if constexpr (L <= 8) {   // per-step factors: latency bound, short chunks
-        if (a.stream) return one ? launch_fx_t<L, true, true, true>(a, ngroups, s)
-                                 : launch_fx_t<L, false, true, true>(a, ngroups, s);
+        if (a.stream) return launch_fx_f<L, true, true, false>(a, one, full, ngroups, s);
     }
     if (a.stream) return -2;
-    if (a.beta) {   // S_0^2 ends: instantiations of their own, so that Robin ones keep their registers
-        if (a.fin) return one ? launch_fx_t<L, true, true, false, true>(a, ngroups, s)
-                              : launch_fx_t<L, false, true, false, true>(a, ngroups, s);
-        return one ? launch_fx_t<L, true, false, false, true>(a, ngroups, s)
-                   : launch_fx_t<L, false, false, false, true>(a, ngroups, s);
-    }
-    if (a.fin) return one ? launch_fx_t<L, true, true, false>(a, ngroups, s)
-                          : launch_fx_t<L, false, true, false>(a, ngroups, s);
-    return one ? launch_fx_t<L, true, false, false>(a, ngroups, s)
-               : launch_fx_t<L, false, false, false>(a, ngroups, s);
+    if (a.beta)   // S_0^2 ends: instantiations of their own, so that Robin ones keep their registers
+        return a.fin ? launch_fx_f<L, true, false, true>(a, one, true, ngroups, s)
+                     : launch_fx_f<L, false, false, true>(a, one, true, ngroups, s);
+    return a.fin ? launch_fx_f<L, true, false, false>(a, one, full, ngroups, s)
+                 : launch_fx_f<L, false, false, false>(a, one, full, ngroups, s);
 }
 
 int swr_launch_fx_start(const FactorSet& fs, FxMarchArgs a, int nsys, const double2* gin,
@@ -1149,6 +1157,7 @@ int swr_launch_fx_flux(const FxMarchArgs& a, int nsys, double2 two_sigma, const 
 // ---------------------------------------------------------------------------
 constexpr int kSupTile = 128;
 
+template <bool FULL>
 __device__ __forceinline__ double2 superpose_side_fx(const FxC* __restrict__ col, size_t stride,
                                                      bool in, const double2* __restrict__ gs,
                                                      int nt, int sc, const int* __restrict__ sh, int4* tile,
@@ -1202,7 +1211,7 @@ __device__ __forceinline__ double2 superpose_side_fx(const FxC* __restrict__ col
                     FxC x;
                     x.r = (fx_int)(((unsigned long long)(unsigned)v[e].y << 32) | (unsigned)v[e].x);
                     x.i = (fx_int)(((unsigned long long)(unsigned)v[e].w << 32) | (unsigned)v[e].z);
-                    fx_mac(c, fx_split(x), tile[q + e]);
+                    fx_mul<FULL>(c, fx_split(x), tile[q + e]);
                 }
                 hr = c.hr + (c.mr >> 32);
                 hi = c.hi + (c.mi >> 32);
@@ -1226,6 +1235,7 @@ __device__ __forceinline__ double2 superpose_side_f64(const double2* __restrict_
     return acc;
 }
 
+template <bool FULL>
 __global__ void __launch_bounds__(256) k_superpose_fx(
     int L, int P, const double2* __restrict__ urec, const long long* __restrict__ rec_base,
     const MarchSys* __restrict__ sys, const int3* __restrict__ subsys,
@@ -1261,7 +1271,7 @@ __global__ void __launch_bounds__(256) k_superpose_fx(
         if (s < 0 || gi < 0) continue;
         const double2* col = base + (size_t)side * nt * rs;
         u = cadd(u, bad[s] ? superpose_side_f64(col + node, n, in, g + gi, nt)
-                           : superpose_side_fx(reinterpret_cast<const FxC*>(col) + e, rs, in, g + gi,
+                           : superpose_side_fx<FULL>(reinterpret_cast<const FxC*>(col) + e, rs, in, g + gi,
                                                nt, scale[s],
                                                shift + ((size_t)s * 2 + side) * ntmax, tile, &mx));
     }
@@ -1273,9 +1283,10 @@ int swr_launch_superpose_fx(const FactorSet& fs, const double2* urec, const long
                             const MarchSys* sys, const int3* subsys, int N, const int* sub_n,
                             const int* sub_goff, const int* sub_tc, const int* scale,
                             const int* shift, int ntmax, const int* bad, const double2* g,
-                            double2* uT, cudaStream_t s) {
+                            double2* uT, int full, cudaStream_t s) {
     dim3 grid(((fs.L + 1) * (fs.P + 1) + 255) / 256, N);
-    k_superpose_fx<<<grid, 256, 0, s>>>(fs.L, fs.P, urec, rec_base, sys, subsys, sub_n, sub_goff,
+    const auto kern = full ? k_superpose_fx<true> : k_superpose_fx<false>;
+    kern<<<grid, 256, 0, s>>>(fs.L, fs.P, urec, rec_base, sys, subsys, sub_n, sub_goff,
                                         sub_tc, fs.sub_P, fs.sep_pos, fs.clen, scale, shift, ntmax,
                                         bad, g, uT);
     swr_count_launch(1);
