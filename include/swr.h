@@ -370,6 +370,23 @@ void swr_destroy(swr_plan_t p);
  * Synchronises the plan's stream. */
 swr_status swr_get_stats(swr_plan_t p, swr_stats *out, int32_t reset);
 
+/* The lists of systems that a plan marches in 64-bit fixed point (see swr_tuning.two_level). */
+typedef enum {
+    SWR_FX_BUILD = 0,       /* swr_build_interface, V(x): zero flux and unit impulses       */
+    SWR_FX_PRECOND = 1,     /* swr_build_interface: the preconditioner's impulses           */
+    SWR_FX_ZERO_FLUX = 2,   /* zero-flux marches alone: V(t,x) build, swr_adjoint           */
+    SWR_FX_R = 3,           /* R g                                                          */
+    SWR_FX_FINAL = 4,       /* the final march of swr_solve                                 */
+    SWR_FX_L = 5            /* L g of the matrix-free method, V(t,x)                        */
+} swr_fx_list;
+
+/* How the last march of a list went (no counterpart in the paper).  *systems: subdomain
+ * systems in it, 0 if the plan marches that list in FP64 or has not marched it yet; *again: those
+ * of them that left the range of the fixed-point march, or whose end traces kept too few bits,
+ * and were marched again in FP64 within the same call.  Either pointer may be NULL (host).
+ * Synchronises the plan's stream.  Errors: SWR_ERR_ARG, SWR_ERR_CUDA. */
+swr_status swr_fixed_point_counts(swr_plan_t p, int32_t list, int64_t *systems, int64_t *again);
+
 /* x = (I - L)^{-1} y by the causal block forward substitution of the CAUSAL
  * preconditioner, WITHOUT allocating device memory.  The paper has no
  * counterpart: this is a deployment variant of swr_apply_precond.

@@ -171,6 +171,7 @@ struct swr_plan_s {
             int start, count, T, C;
         };
         std::vector<Launch> launches;
+        mutable bool ran = false;
     };
     FxList fx_build, fx_imp, fx_d, fx_R, fx_final, fx_L;
     std::vector<cudaStream_t> fx_side;   // launches of a list beside the first
@@ -727,6 +728,7 @@ swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxL
             rc = -1;
     }
     if (!rc) rc = swr_launch_fx_flux(a, fl.nsys, p->two_sigma, gin, gout, trace, p->s);
+    fl.ran = true;
     again.only = fl.d_bad;
     again.record = record;
     if (!rc)
@@ -2608,6 +2610,21 @@ swr_status swr_solve(swr_plan_t p, double* g_, int32_t g_is_initial, double* uT_
     if (info) *info = loc;
     p->solved = (st == SWR_OK);
     return st;
+}
+
+swr_status swr_fixed_point_counts(swr_plan_t p, int32_t list, int64_t* systems, int64_t* again) {
+    if (!p || list < SWR_FX_BUILD || list > SWR_FX_L) return SWR_ERR_ARG;
+    const swr_plan_s::FxList* all[] = {&p->fx_build, &p->fx_imp, &p->fx_d, &p->fx_R, &p->fx_final, &p->fx_L};
+    const swr_plan_s::FxList& fl = *all[list];
+    if (systems) *systems = 0;
+    if (again) *again = 0;
+    if (!fl.ran) return SWR_OK;
+    std::vector<int> bad(fl.nsys);
+    CK(cudaMemcpyAsync(bad.data(), fl.d_bad, sizeof(int) * fl.nsys, cudaMemcpyDeviceToHost, p->s));
+    CK(cudaStreamSynchronize(p->s));
+    if (systems) *systems = fl.nsys;
+    if (again) *again = fl.nsys - std::count(bad.begin(), bad.end(), 0);
+    return SWR_OK;
 }
 
 swr_status swr_apply_R(swr_plan_t p, const double* g_in, double* g_out) {

@@ -135,6 +135,8 @@ def lib():
         L.swr_fp64_peak.argtypes = [ctypes.c_int32, ctypes.c_int64, ctypes.c_int32,
                                     ctypes.c_int32, dp, ctypes.POINTER(ctypes.c_double),
                                     ctypes.POINTER(ctypes.c_float), vp]
+        L.swr_fixed_point_counts.argtypes = [vp, ctypes.c_int32, ctypes.POINTER(ctypes.c_int64),
+                                             ctypes.POINTER(ctypes.c_int64)]
         L.swr_test_wait_hook.argtypes = [ctypes.c_int64, ctypes.c_int32]
         L.swr_destroy.argtypes = [vp]
         L.swr_destroy.restype = None
@@ -145,7 +147,7 @@ def lib():
         for f in ("swr_plan", "swr_plan_batch", "swr_plan_ex", "swr_plan_batch_ex",
                   "swr_build_interface", "swr_solve", "swr_apply_R",
                   "swr_apply_interface", "swr_get_interface", "swr_apply_precond", "swr_adjoint",
-                  "swr_get_stats", "swr_causal_solve_noalloc", "swr_misfit", "swr_fp64_peak",
+                  "swr_get_stats", "swr_fixed_point_counts", "swr_causal_solve_noalloc", "swr_misfit", "swr_fp64_peak",
                   "swr_test_wait_hook"):
             getattr(L, f).restype = ctypes.c_int
         _lib = L
@@ -306,6 +308,17 @@ class Plan:
         st = swr_stats()
         _check(lib().swr_get_stats(self.handle, ctypes.byref(st), int(bool(reset))), "swr_get_stats")
         return st.as_dict()
+
+    def fixed_point_counts(self):
+        """{list: (systems, again)} of the last march of every list of fixed-point marches
+        (swr_fixed_point_counts): build, precond, zero_flux, R, final, L."""
+        out = {}
+        for k, name in enumerate(("build", "precond", "zero_flux", "R", "final", "L")):
+            n, b = ctypes.c_int64(), ctypes.c_int64()
+            _check(lib().swr_fixed_point_counts(self.handle, k, ctypes.byref(n), ctypes.byref(b)),
+                   "swr_fixed_point_counts")
+            out[name] = (n.value, b.value)
+        return out
 
     def destroy(self):
         if getattr(self, "handle", None):
