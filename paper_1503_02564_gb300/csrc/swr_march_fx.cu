@@ -180,7 +180,13 @@ __device__ __forceinline__ FxSub fx_sub(const unsigned long long* mx, double his
             g2 *= 1.0 + get(B_RG + k);
             bad |= get(B_PG + k) > 2.6 || get(B_RG + k) > 2.6;
         }
-        bad |= get(B_CO) > 1.1 || get(B_AX) > 2.6 || get(B_Y) > 4.0;
+        // x of the backward sweep: B_Y from the right-hand sides, and from vL and vR at most 1.42
+        // for any grid (V = 0; 2.5 taken), 8 in all, |x| < 2^61.  B_Y overestimates by up to a
+        // quarter: 4.25 at most for exact moduli, up to 5.3 from the recurrences of k_fx_bounds,
+        // where dt/h^2 is about 0.2 or, with 12 nodes and more, 3 to 10.  (The limit was 4: all
+        // marches of such a grid ran in FP64 in an untuned shape, a solve of 1355 nodes and 372
+        // steps in 12.7 ms instead of 5.2.)
+        bad |= get(B_CO) > 1.1 || get(B_AX) > 2.6 || get(B_Y) > 5.5;
         // a separator's row: its stencil and a flux, the two chunks' parts
         // (and with S_0^2 ends a history term of a few times |c2 / (i kappa)| v, tested as it comes)
         const double d0 = 2.0 * kFxF + get(B_D) + get(B_CZ) + 6.0 * hist;

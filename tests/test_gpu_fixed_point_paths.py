@@ -187,3 +187,24 @@ def test_streamed_state_scaled_down(chunk, sizes):
     wl = moving(workload(sizes, 64))
     g = W.random_interface(wl.nblk, wl.nt, 52) * (2.0 ** (40.0 * np.arange(wl.nt) / wl.nt))
     check_streamed(wl, chunk, 0, g)
+
+
+# ---- factors within the range ------------------------------------------------------------
+@pytest.mark.parametrize("nx,h,nt,nsub", [(1355, 24 / 1354, 372, 4), (862, 1.6e-2, 150, 3),
+                                          (1700, 24 / 1699, 300, 5), (278, 24 / 277, 473, 6),
+                                          (420, 24 / 419, 400, 6)])
+@pytest.mark.parametrize("chunk", [0, 4, 8, 12])
+def test_coarse_grids_stay_in_fixed_point(nx, h, nt, nsub, chunk):
+    """Grids on which the chunks' solutions are largest against their right-hand sides."""
+    base, extra = divmod(nx - 1, nsub)
+    wl = workload([base + (j < extra) for j in range(nsub)], nt, h)
+    wl.V = -wl.x ** 2 / 4
+    plan = make(wl, chunk)
+    d, cols = interface(plan)
+    assert plan.fixed_point_counts()["build"] == (3 * nsub - 2, 0)
+    r = apply_R(plan, W.random_interface(wl.nblk, wl.nt, 63))
+    assert plan.fixed_point_counts()["R"] == (nsub, 0)
+    plan.destroy()
+    P = problem(wl)
+    assert rel(d, O.build_d(P)) < TOL_MARCH and rel(cols, O.build_columns(P)) < TOL_MARCH
+    assert rel(r, O.apply_R(P, W.random_interface(wl.nblk, wl.nt, 63))) < TOL_MARCH
