@@ -208,3 +208,28 @@ def test_coarse_grids_stay_in_fixed_point(nx, h, nt, nsub, chunk):
     P = problem(wl)
     assert rel(d, O.build_d(P)) < TOL_MARCH and rel(cols, O.build_columns(P)) < TOL_MARCH
     assert rel(r, O.apply_R(P, W.random_interface(wl.nblk, wl.nt, 63))) < TOL_MARCH
+
+
+# ---- nothing of the build is put off -----------------------------------------------------
+@pytest.mark.parametrize("nx,nsub", [(48015, 80), (22190, 3), (20543, 11), (159333, 18)])
+@pytest.mark.parametrize("tc", [0, 1])
+def test_first_march_after_a_build_is_like_the_next(nx, nsub, tc):
+    """R g launches the same kernels right after a build as later: its factors are the build's."""
+    from paper_1503_02564_gb300 import swr
+    base, extra = divmod(nx - 1, nsub)
+    wl = workload([base + (j < extra) for j in range(nsub)], 40)
+    plan = swr.Plan(nx=wl.nx, a0=wl.a0, b0=wl.b0, nt=wl.nt, dt=wl.dt, nsub=wl.nsub, node_off=wl.off,
+                    p=wl.sigma, tc=tc)
+    g = W.random_interface(wl.nblk, wl.nt, 64)
+    launches, out = [], []
+    for k in range(3):
+        if k < 2:
+            plan.build_interface(dev(wl.V * (1.0 + k)), dev(wl.u0))
+        n0 = swr.swr_kernel_launch_count()
+        out.append(apply_R(plan, g))
+        launches.append(swr.swr_kernel_launch_count() - n0)
+    plan.destroy()
+    assert launches[0] == launches[1] == launches[2]
+    assert np.array_equal(out[1], out[2])
+    wl.V = wl.V * 2.0
+    assert rel(out[1], O.apply_R(problem(wl, tc), g)) < TOL_MARCH
