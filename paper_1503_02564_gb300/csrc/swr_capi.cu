@@ -956,6 +956,18 @@ swr_status assemble(swr_plan_t p, const double* V, double2* dg, double2* od) {
     return SWR_OK;
 }
 
+// Offsets of the recorded states per subdomain (Phi_l, Phi_r: nt x rec_n, U_d: n); their total.
+long long record_layout(const swr_plan_s* p, std::vector<long long>& base) {
+    long long tot = 0;
+    base.assign(p->N, 0);
+    for (const InstInfo& I : p->inst)
+        for (int j = 0; j < I.N; ++j) {
+            base[I.sub0 + j] = tot;
+            tot += 2LL * I.nt * p->rec_n[I.sub0 + j] + p->n[I.sub0 + j];
+        }
+    return tot;
+}
+
 // March systems of every instance.  Flux offsets are absolute (complex entries):
 // an instance's interface blocks (2N-2 of nt) start at its foff, block 2k = r_k,
 // 2k+1 = l_{k+1}; its first columns start at nb + coff in the build buffer
@@ -2051,13 +2063,8 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
         // u(T) by superposition: Phi_l, Phi_r (nt x n_j each) and U_d per subdomain, if
         // they take at most a quarter of the free memory
         const bool on = p->tune.superpose >= 0;
-        long long tot = 0;
-        std::vector<long long> base(p->N, 0);
-        for (const InstInfo& I : p->inst)
-            for (int j = 0; j < I.N; ++j) {
-                base[I.sub0 + j] = tot;
-                tot += 2LL * I.nt * p->rec_n[I.sub0 + j] + p->n[I.sub0 + j];
-            }
+        std::vector<long long> base;
+        const long long tot = record_layout(p, base);
         size_t fr = 0, all = 0;
         if (on && cudaMemGetInfo(&fr, &all) == cudaSuccess &&
             (size_t)tot * sizeof(double2) <= fr / 4 && dalloc(&p->d_urec, (size_t)tot) == SWR_OK &&
@@ -2274,17 +2281,16 @@ static swr_status build_body(swr_plan_t p, bool do_assemble) {
         if (fx) LK(swr_launch_fx_prepare(p->fsL[lidx(Lb)], p->N, s, 0, 1, p->fx_hist));
         // the factors of R g, where the build marches in FP64, beside those marches (22190 nodes in
         // 3 subdomains, 79 steps: a build of 2.05 ms with them, 2.05 without, 2.13 in one stream)
-        const bool side = p->fx_R.sys && p->fac_side;
+        const bool own = p->fx_R.sys && !fx, side = own && p->fac_side;
+        cudaStream_t sr = side ? p->fac_side : s;
         if (side) {
             CK(cudaEventRecord(p->fac_fork, s));
-            CK(cudaStreamWaitEvent(p->fac_side, p->fac_fork, 0));
-            if (La != Lb && (st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od, p->fac_side)))
-                return st;
-            LK(swr_launch_fx_prepare(p->fsL[lidx(La)], p->N, p->fac_side, 0, 1, p->fx_hist));
-            CK(cudaEventRecord(p->fac_join, p->fac_side));
-        } else if (La != Lb && (st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od))) {
-            return st;
+            CK(cudaStreamWaitEvent(sr, p->fac_fork, 0));
         }
+        if (La != Lb && (st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od, sr)))
+            return st;
+        if (own) LK(swr_launch_fx_prepare(p->fsL[lidx(La)], p->N, sr, 0, 1, p->fx_hist));
+        if (side) CK(cudaEventRecord(p->fac_join, sr));
         CK(cudaMemsetAsync(p->d_iface, 0, sizeof(double2) * (nb + (size_t)p->ncols), s));
         // Algorithm 3, step 1: d and the first columns, 3 marches per interior subdomain
         st = run_march(p, false, p->d_sys_build, p->nsys_build, nullptr, p->d_iface, nullptr,
@@ -2325,6 +2331,94 @@ static swr_status build_body(swr_plan_t p, bool do_assemble) {
             LK(swr_launch_col_spectra(p->N, p->nt, p->d_iface0 + nb, p->d_spec0, p->fftM,
                                       p->d_W, s, p->batched ? p->d_inst : nullptr, p->ninst));
         p->have_L0 = true;
+    }
+    return SWR_OK;
+}
+
+// After the first build, with autotuning: a list some of whose systems went back to FP64 marches
+// those after the others, which can take longer than all of them in FP64 at a measured shape
+// (200001 nodes, 500 steps, one subdomain of 16 out of range: 27.1 ms for the build, in FP64 20.2).
+// Both are timed once and the faster stays; *changed: the build's outputs have to be formed anew.
+static swr_status fx_settle(swr_plan_t p, bool* changed) {
+    struct Case {
+        swr_plan_s::FxList* fl;
+        bool zero;
+        const MarchSys* sys;
+        int nsys;
+        double2* out;
+        long long work;
+    };
+    const Case cases[] = {
+        {&p->fx_build, false, p->d_sys_build, p->nsys_build, p->d_iface, p->work_build},
+        {&p->fx_imp, true, p->d_sys_build + p->N, p->nsys_build - p->N, p->d_iface0, p->work_build_imp}};
+    // V(t,x): a step out of range takes every march of its subdomain back to FP64
+    if (p->fx_tdep && p->fx_d.ran) {
+        int64_t again = 0;
+        swr_status st = swr_fixed_point_counts(p, SWR_FX_ZERO_FLUX, nullptr, &again);
+        if (st) return st;
+        bool out = false;
+        if (again) {
+            const FactorSet& fs = p->fsL[lidx(p->fx_R.sh.L)];
+            std::vector<FxSub> sub((size_t)p->nt * p->N);
+            CK(cudaMemcpy(sub.data(), fs.fx_sub, sizeof(FxSub) * sub.size(), cudaMemcpyDeviceToHost));
+            for (const FxSub& f : sub) out = out || f.bad;
+        }
+        if (out) {
+            p->fx_tdep = p->fx_d.ran = false;
+            p->tuned.erase(std::remove_if(p->tuned.begin(), p->tuned.end(),
+                                          [](const auto& t) { return t[0] == MK_TSTAT; }),
+                           p->tuned.end());
+            if ((st = tune_march(p, MK_TSTAT, false, p->d_sys_R, p->N, p->d_iface, p->d_V, p->d_dg, p->d_od)))
+                return st;
+            *changed = true;
+        }
+    }
+    for (const Case& c : cases) {
+        if (!c.fl->sys || !c.fl->ran) continue;
+        int64_t again = 0;
+        swr_status st = swr_fixed_point_counts(p, c.zero ? SWR_FX_PRECOND : SWR_FX_BUILD, nullptr, &again);
+        if (st) return st;
+        if (!again) continue;
+        cudaEvent_t e0, e1;
+        CK(cudaEventCreate(&e0));
+        CK(cudaEventCreate(&e1));
+        float ms[2] = {0.f, 0.f};
+        const MarchSys* was = c.fl->sys;
+        const double* V = c.zero ? (p->d.precond == SWR_PC_MEAN_POTENTIAL ? p->d_Vbar : nullptr) : p->d_V;
+        double2 *dg = c.zero ? p->d_dg0 : p->d_dg, *od = c.zero ? p->d_od0 : p->d_od;
+        for (int k = 0; k < 2 && !st; ++k) {
+            if (k == 1) {
+                c.fl->sys = nullptr;
+                st = tune_march(p, MK_STATIC, c.zero, c.sys, c.nsys, c.out, V, dg, od);
+                const int L = march_config(p, c.nsys).L;
+                if (!st) st = factor_for(p, c.zero ? p->fs0L[lidx(L)] : p->fsL[lidx(L)], L, V, dg, od);
+            }
+            if (!st && cudaEventRecord(e0, p->s) != cudaSuccess) st = SWR_ERR_CUDA;
+            if (!st)
+                st = run_march(p, c.zero, c.sys, c.nsys, nullptr, c.out, nullptr, nullptr, p->d_u0, c.work);
+            if (!st && (cudaEventRecord(e1, p->s) != cudaSuccess || cudaEventSynchronize(e1) != cudaSuccess ||
+                        cudaEventElapsedTime(&ms[k], e0, e1) != cudaSuccess))
+                st = SWR_ERR_CUDA;
+        }
+        cudaEventDestroy(e0);
+        cudaEventDestroy(e1);
+        if (st) return st;
+        *changed = true;   // the timed marches wrote into the outputs
+        if (ms[1] >= ms[0]) {
+            c.fl->sys = was;
+            continue;
+        }
+        c.fl->ran = false;
+        if (!c.zero && p->superpose) {   // the FP64 marches' records: local node order
+            p->rec_n = p->n;
+            record_layout(p, p->rec_base);
+            const auto vb = build_systems(p, true);
+            CK(cudaMemcpy(p->d_rec_base, p->rec_base.data(), sizeof(long long) * p->N, cudaMemcpyHostToDevice));
+            CK(cudaMemcpy(p->d_sys_build, vb.data(), sizeof(MarchSys) * vb.size(), cudaMemcpyHostToDevice));
+        }
+        if (p->tune.debug >= 1)
+            fprintf(stderr, "swr: %lld of %d systems out of fixed point's range, list in FP64 (%.3f ms, %.3f)\n",
+                    (long long)again, c.nsys, ms[1], ms[0]);
     }
     return SWR_OK;
 }
@@ -2457,6 +2551,16 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
     CK(cudaEventRecord(p->ev[1], s));
     st = read_status(p);
     if (st) return st;
+    if (!p->built && p->autotune) {
+        bool changed = false;
+        if ((st = fx_settle(p, &changed))) return st;
+        if (changed) {   // the same build with the FP64 marches
+            CK(cudaEventRecord(p->ev[0], s));
+            if ((st = build_body(p, false))) return st;
+            CK(cudaEventRecord(p->ev[1], s));
+            if ((st = read_status(p))) return st;
+        }
+    }
     if (!p->built && p->auto_sweeps) {
         // The substitution's same-step coupling of neighbouring interfaces is the
         // corner entries cB_k = X^{k+1,2}[0], cD_k = X^{k,3}[0] of the subdomain

@@ -233,3 +233,46 @@ def test_first_march_after_a_build_is_like_the_next(nx, nsub, tc):
     assert np.array_equal(out[1], out[2])
     wl.V = wl.V * 2.0
     assert rel(out[1], O.apply_R(problem(wl, tc), g)) < TOL_MARCH
+
+
+# ---- lists that are faster in FP64 -------------------------------------------------------
+def test_list_with_flagged_systems_settles_in_fp64():
+    """One subdomain of eight out of range: the second march, which only starts when the others
+    are done, takes the build past its time in FP64 (4.5 against 2.9 ms), so the first build
+    settles on FP64.  Later builds (the third is replayed from the graph) and solves agree."""
+    from paper_1503_02564_gb300 import swr
+    wl = workload([2500] * 8, 200, inside=3, value=1e6)
+    plan = swr.Plan(nx=wl.nx, a0=wl.a0, b0=wl.b0, nt=wl.nt, dt=wl.dt, nsub=wl.nsub, node_off=wl.off,
+                    p=wl.sigma, precond=swr.SWR_PC_CAUSAL)
+    P = problem(wl)
+    dr, cr, (gs, uTm) = O.build_d(P), O.build_columns(P), O.mono_interface(P)
+    g = W.random_interface(wl.nblk, wl.nt, 65)
+    rr = O.apply_R(P, g)
+    for k in range(3):
+        plan.build_interface(dev(wl.V), dev(wl.u0))
+        assert plan.fixed_point_counts()["build"] == (0, 0)
+        d, cols = interface(plan)
+        uT = torch.zeros(wl.nx, dtype=torch.complex128, device="cuda")
+        gx = torch.zeros(plan.n_interface, dtype=torch.complex128, device="cuda")
+        plan.solve(gx, False, uT)
+        assert rel(d, dr) < TOL_MARCH and rel(cols, cr) < TOL_MARCH
+        assert rel(apply_R(plan, g), rr) < TOL_MARCH
+        assert rel(uT.cpu().numpy(), uTm) < TOL_SOLVE and rel(gx.cpu().numpy(), gs) < TOL_SOLVE
+    assert plan.get_stats()["superposed"] == 1
+    plan.destroy()
+
+
+def test_streamed_list_with_flagged_systems_settles_in_fp64():
+    from paper_1503_02564_gb300 import swr
+    wl = moving(workload([400, 390, 410], 40), (20, 1, 4e6))
+    plan = swr.Plan(nx=wl.nx, a0=wl.a0, b0=wl.b0, nt=wl.nt, dt=wl.dt, nsub=wl.nsub, node_off=wl.off,
+                    p=wl.sigma, vkind=swr.SWR_V_TIME)
+    P = problem(wl)
+    g = W.random_interface(wl.nblk, wl.nt, 66)
+    for k in range(3):
+        plan.build_interface(dev(wl.V), dev(wl.u0))
+        assert plan.fixed_point_counts()["zero_flux"] == (0, 0)
+        assert rel(interface(plan)[0], O.build_d(P)) < TOL_MARCH
+        assert rel(apply_R(plan, g), O.apply_R(P, g)) < TOL_MARCH
+        assert plan.fixed_point_counts()["R"] == (0, 0)
+    plan.destroy()
