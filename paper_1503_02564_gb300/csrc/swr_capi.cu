@@ -180,6 +180,7 @@ struct swr_plan_s {
     cudaStream_t fac_side = nullptr;     // R g in fixed point, the build in FP64: R g's factors
     cudaEvent_t fac_fork = nullptr, fac_join = nullptr;
     bool fx_full = false;                // whole products (see plan_create)
+    bool fx_tdep_asked = false;          // they were to have one
     bool fx_tdep = false;                // V(t,x): the per-step factors have a fixed-point form
     bool fac_stale[5] = {};              // fsL[] of another chunk length than the last build's
     int3* d_subsys = nullptr;            // per subdomain: its systems in the build list
@@ -2351,27 +2352,29 @@ static swr_status fx_settle(swr_plan_t p, bool* changed) {
     const Case cases[] = {
         {&p->fx_build, false, p->d_sys_build, p->nsys_build, p->d_iface, p->work_build},
         {&p->fx_imp, true, p->d_sys_build + p->N, p->nsys_build - p->N, p->d_iface0, p->work_build_imp}};
-    // V(t,x): a step out of range takes every march of its subdomain back to FP64
+    // V(t,x): a step out of range takes every march of its subdomain back to FP64, and without room
+    // for the fixed-point rows (fx_tdep gone again) all march there: at the chunk length measured
+    // for FP64, not the one taken for fixed point
+    bool out = p->fx_tdep_asked && !p->fx_tdep;
     if (p->fx_tdep && p->fx_d.ran) {
         int64_t again = 0;
         swr_status st = swr_fixed_point_counts(p, SWR_FX_ZERO_FLUX, nullptr, &again);
         if (st) return st;
-        bool out = false;
         if (again) {
             const FactorSet& fs = p->fsL[lidx(p->fx_R.sh.L)];
             std::vector<FxSub> sub((size_t)p->nt * p->N);
             CK(cudaMemcpy(sub.data(), fs.fx_sub, sizeof(FxSub) * sub.size(), cudaMemcpyDeviceToHost));
             for (const FxSub& f : sub) out = out || f.bad;
         }
-        if (out) {
-            p->fx_tdep = p->fx_d.ran = false;
-            p->tuned.erase(std::remove_if(p->tuned.begin(), p->tuned.end(),
-                                          [](const auto& t) { return t[0] == MK_TSTAT; }),
-                           p->tuned.end());
-            if ((st = tune_march(p, MK_TSTAT, false, p->d_sys_R, p->N, p->d_iface, p->d_V, p->d_dg, p->d_od)))
-                return st;
-            *changed = true;
-        }
+    }
+    if (out) {
+        p->fx_tdep = p->fx_tdep_asked = p->fx_d.ran = false;
+        p->tuned.erase(std::remove_if(p->tuned.begin(), p->tuned.end(),
+                                      [](const auto& t) { return t[0] == MK_TSTAT; }),
+                       p->tuned.end());
+        swr_status st = tune_march(p, MK_TSTAT, false, p->d_sys_R, p->N, p->d_iface, p->d_V, p->d_dg, p->d_od);
+        if (st) return st;
+        *changed = true;
     }
     for (const Case& c : cases) {
         if (!c.fl->sys || !c.fl->ran) continue;
@@ -2455,13 +2458,13 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
         }
         p->tdep_pre = on ? 1 : 0;
         if (on && p->fx_R.sys) {
-            // the fixed-point form beside them: another set of the same size, within a quarter
-            // of the free memory
+            // the fixed-point form beside them, another set of the same size: both within that half
             size_t fr = 0, tot = 0;
             CK(cudaMemGetInfo(&fr, &tot));
             const int L = p->fx_R.sh.L, P = chunks_for(p->nmax, L);
             const size_t fac = (size_t)p->nt * swr_factor_step_bytes(p->N, L, P);
-            p->fx_tdep = fac <= fr / 2 && (size_t)p->nt * swr_fx_step_bytes(p->N, L, P) <= fr / 4;
+            p->fx_tdep = fac + (size_t)p->nt * swr_fx_step_bytes(p->N, L, P) <= fr / 2;
+            p->fx_tdep_asked = p->fx_tdep;
             if (p->fx_tdep && !p->autotune) {   // one chunk length for both forms
                 const MarchCfg c = march_config(p, p->N, MK_TSTAT, L);
                 p->tuned.push_back({MK_TSTAT, p->N, c.L, c.C, c.G, c.T, c.ngroups, c.ragged});
