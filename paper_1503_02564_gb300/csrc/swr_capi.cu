@@ -17,6 +17,7 @@
 
 #include <nvtx3/nvToolsExt.h>   // header-only; the ranges cost nothing without a tool attached
 
+#include "swr_fx.cuh"
 #include "swr_internal.cuh"
 
 static std::atomic<long long> g_launches{0};
@@ -2137,18 +2138,11 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
                               cudaMemcpyHostToDevice) != cudaSuccess)
             st = SWR_ERR_CUDA;
         if (!st && d->tc == SWR_TC_S02 && (fx || fx_one)) {
-            auto limbs = [](double c) {   // rint(c 2^61)
-                const long long C = (long long)std::llrint(std::ldexp(c, 61));
-                const int l = (int)(uint32_t)(uint64_t)C;
-                return make_int2((int)((C - l) >> 32), l);
-            };
             std::vector<int2> bl(p->nt + 1);
-            for (int k = 0; k <= p->nt; ++k) bl[k] = limbs(beta[k]);
+            for (int k = 0; k <= p->nt; ++k) bl[k] = fx_limbs(beta[k]);
             p->fx_hist = std::hypot(p->c2_ik.x, p->c2_ik.y);
             p->fx_c2e = std::ilogb(p->fx_hist) + 1;
-            const int2 re = limbs(std::ldexp(p->c2_ik.x, -p->fx_c2e));
-            const int2 im = limbs(std::ldexp(p->c2_ik.y, -p->fx_c2e));
-            p->fx_c2 = make_int4(re.x, re.y, im.x, im.y);
+            p->fx_c2 = fx_coef(std::ldexp(p->c2_ik.x, -p->fx_c2e), std::ldexp(p->c2_ik.y, -p->fx_c2e));
             st = dalloc(&p->d_fxbeta, bl.size());
             if (!st && cudaMemcpy(p->d_fxbeta, bl.data(), sizeof(int2) * bl.size(),
                                   cudaMemcpyHostToDevice) != cudaSuccess)

@@ -27,6 +27,7 @@
 
 #include <limits.h>
 #include <stdint.h>
+#include <string.h>
 
 typedef long long fx_int;
 
@@ -169,19 +170,20 @@ __device__ __forceinline__ void fx_mac_pow2(FxAcc& a, FxS x, int ch) {
     a.mi = fx_mw(x.il, ch, a.mi);
 }
 // limbs of a coefficient
-__device__ __forceinline__ int2 fx_limbs(double c) {
+__host__ __device__ __forceinline__ int2 fx_limbs(double c) {
     // rint(c 2^61) from the bits of c (ties away from zero): a conversion instruction and the
     // scaling before it cost 64 cycles each
-    const fx_int b = __double_as_longlong(c);
+    fx_int b;
+    memcpy(&b, &c, sizeof b);
     const int e = (int)((b >> 52) & 0x7ff) - 1023 + 61 - 52;      // c = m 2^(e - 61)
     const fx_int m = (b & 0xfffffffffffffLL) | (e > -1023 + 61 - 52 ? 0x10000000000000LL : 0);
-    fx_int C = e >= 0 ? m << min(e, 10) : (e > -54 ? ((m >> (-e - 1)) + 1) >> 1 : 0);
+    fx_int C = e >= 0 ? m << (e < 10 ? e : 10) : (e > -54 ? ((m >> (-e - 1)) + 1) >> 1 : 0);
     if (b < 0) C = -C;
     C += (int)C == INT_MIN;   // its low limb has a negative (see fx_mac)
     const int l = (int)C;
     return make_int2((int)((C - l) >> 32), l);
 }
-__device__ __forceinline__ int4 fx_coef(double re, double im) {
+__host__ __device__ __forceinline__ int4 fx_coef(double re, double im) {
     const int2 a = fx_limbs(re), b = fx_limbs(im);
     return make_int4(a.x, a.y, b.x, b.y);
 }
