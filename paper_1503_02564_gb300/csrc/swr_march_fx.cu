@@ -500,7 +500,9 @@ __device__ __forceinline__ FxC fx_history(const int2* __restrict__ beta, FxC v0,
         mr += __shfl_xor_sync(0xffffffffu, mr, off);
         mi += __shfl_xor_sync(0xffffffffu, mi, off);
     }
-    // (H 2^64 + M 2^32) / 2^61 / 2^kFxHist: sum |beta_s| < 36 for 2048 steps, so that |4 H| < 2^63
+    // (H 2^64 + M 2^32) / 2^61 / 2^kFxHist.  sum |beta_s| < 72 for 2048 steps and |v| < 2^58, so
+    // that a sum may reach 1.12 2^63; one that wraps is then below -2^60 or above 2^60, where the
+    // march's range check of the history flags the system.  (H itself stays below 2^62.)
     constexpr int e = 29 + kFxHist;
     const fx_int half = (fx_int)1 << (e - 1);
     const FxC a = {(hr << (3 - kFxHist)) + ((mr + half) >> e), (hi << (3 - kFxHist)) + ((mi + half) >> e)};

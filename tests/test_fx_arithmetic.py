@@ -55,3 +55,17 @@ def test_limbs(convert):
             assert -2 ** 31 < low < 2 ** 31 and -2 ** 31 < h < 2 ** 31
             num, den = c.as_integer_ratio()
             assert abs((h * 2 ** 32 + low) * den - num * 2 ** 61) <= den + den // 2   # rounding, and one unit
+
+
+def test_history_sums_that_wrap_are_out_of_range():
+    """sum |beta_s| over 2047 lags is 71.3, the traces stay below 2^58: a history sum in units of 2
+    may reach 2^63.2 and wrap.  A wrapped one lies outside the 2^60 at which it is flagged."""
+    a, total = 1.0, 0.0
+    for k in range(0, 2048, 2):
+        total += a + (a if k else 0.0)      # beta_0 belongs to the current step
+        a *= (k + 1) / (k + 2)
+    assert total < 72
+    top = int(total * 2 ** 58) // 2
+    assert 2 ** 63 < top < 2 ** 64 - 2 ** 60     # wrapped: from top - 2^64 to -2^63, all below -2^60
+    for s in (2 ** 63, top, (2 ** 63 + top) // 2):
+        assert abs(((s + 2 ** 63) % 2 ** 64) - 2 ** 63) >= 2 ** 60
