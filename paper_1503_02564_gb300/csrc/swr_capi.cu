@@ -178,7 +178,11 @@ struct swr_plan_s {
     std::vector<cudaStream_t> fx_side;   // launches of a list beside the first
     cudaEvent_t fx_fork = nullptr;
     std::vector<cudaEvent_t> fx_join;
-    cudaStream_t fac_side = nullptr;     // R g in fixed point, the build in FP64: R g's factors
+    // R g in fixed point, the build in FP64: R g's factors and matrix (see form_R)
+    FactorSet fsR;
+    double2 *d_dgR = nullptr, *d_odR = nullptr;
+    bool uses_R = false, have_R = false;
+    cudaStream_t fac_side = nullptr;
     cudaEvent_t fac_fork = nullptr, fac_join = nullptr;
     bool fx_full = false;                // whole products (see plan_create)
     bool fx_tdep_asked = false;          // they were to have one
@@ -401,6 +405,7 @@ struct SegArgs {
     double *gint = nullptr, *gl = nullptr, *gr = nullptr;
     double2* urec = nullptr;        // recorded states (NULL: the plan's)
     bool record = true;             // false: record no states
+    const FactorSet* fs = nullptr;  // factors (NULL: the plan's of the shape's chunk length)
     const int* only = nullptr;      // march only the flagged systems
     int tstride = 0;                // entries per trace (0: the launch's own step count)
 };
@@ -552,7 +557,7 @@ int launch_cfg(swr_plan_t p, const MarchCfg& cfg, int kind, bool zero_potential,
                const MarchSys* d_sys, int nsys, const double2* gin, double2* gout, double2* uT,
                double2* trace, const double2* u0, int nt_run, const SegArgs& seg = SegArgs()) {
     if (cfg.C > 16) return -2;
-    const FactorSet& fs = zero_potential ? p->fs0L[lidx(cfg.L)] : p->fsL[lidx(cfg.L)];
+    const FactorSet& fs = seg.fs ? *seg.fs : zero_potential ? p->fs0L[lidx(cfg.L)] : p->fsL[lidx(cfg.L)];
     if (fs.L != cfg.L) return -3;
     MarchArgs a{};
     a.nt = nt_run;
@@ -642,26 +647,52 @@ inline int march_kind(swr_plan_t p, bool zero_potential) {
     return MK_STATIC;
 }
 
+swr_status factor_for(swr_plan_t p, FactorSet& fs, int L, const double* V, double2* dg,
+                      double2* od, cudaStream_t s = nullptr);
+
+// R g's own factors.  The plan's first march of R g forms them, and from then on every build does:
+// beside its marches, on a stream of their own with a matrix of their own, after fac_fork (the
+// potential is in the plan); the next build and the marches of R g wait for fac_join.  (A plan
+// that never marches R g, as a solve by GMRES does not, would pay 8 us a build beside the
+// marches, 60 to 80 in the plan's stream: a build of 241 nodes takes 333 us.)
+swr_status form_R(swr_plan_t p, cudaStream_t s) {
+    if (swr_launch_assemble_static(p->d_V, p->N, p->d_n, p->d_goff, p->d_loff, p->d_tc, p->nmax, p->h,
+                                   p->d.dt, p->sigma0, p->inv_ik, p->d_dgR, p->d_odR, s) != 0)
+        return launch_fail("assembly (R g)", __LINE__);
+    swr_status st = factor_for(p, p->fsR, p->fx_R.sh.L, p->d_V, p->d_dgR, p->d_odR, s);
+    if (st) return st;
+    LK(swr_launch_fx_prepare(p->fsR, p->N, s, 0, 1, p->fx_hist));
+    p->have_R = p->uses_R = true;
+    return SWR_OK;
+}
+
 // The fixed-point form of a list's marches: step 1 in FP64 (it sets each system's scale), steps
 // 2..nt in fixed point, the fluxes from the end traces, and the flagged systems again in FP64.
 swr_status run_march_fx(swr_plan_t p, bool zero_potential, const swr_plan_s::FxList& fl,
                         const double2* gin, double2* gout, double2* uT, double2* trace,
                         const double2* u0, long long work, bool record) {
     const int L = fl.sh.L;
-    FactorSet& fs = zero_potential ? p->fs0L[lidx(L)] : p->fsL[lidx(L)];
+    const bool own = !zero_potential && fl.R == 1 && p->fsR.L;
+    FactorSet& fs = own ? p->fsR : (zero_potential ? p->fs0L[lidx(L)] : p->fsL[lidx(L)]);
     if (fs.L != L) return SWR_ERR_STATE;
     const bool steps = fs.nsteps > 1;   // per-step factors
     const int kind = steps ? MK_TSTAT : MK_STATIC;
     const MarchCfg cfg = steps ? march_config(p, fl.nsys, kind) : march_config(p, fl.nsys, kind, L);
-    const int pi = prof_begin(p, 0, work);
     int rc = 0;
     SegArgs first, again;
     first.urec = p->d_fxu;
     first.tstride = p->nt;
+    if (own) {
+        first.fs = again.fs = &p->fsR;
+        CK(cudaStreamWaitEvent(p->s, p->fac_join, 0));
+        swr_status st = p->have_R ? SWR_OK : form_R(p, p->s);
+        if (st) return st;
+    }
     if (p->cur_rev && steps) {   // time-reversed problem: last step's factors first
         first.fstep0 = again.fstep0 = p->nt - 1;
         first.frev = again.frev = 1;
     }
+    const int pi = prof_begin(p, 0, work);
     if (!rc)
         rc = launch_cfg(p, cfg, kind, zero_potential, fl.d_sys1, fl.nsys, gin, gout, nullptr,
                         trace, u0, 1, first);
@@ -762,7 +793,7 @@ swr_status run_march(swr_plan_t p, bool zero_potential, const MarchSys* d_sys, i
 
 // Assemble A - B for V (NULL: V = 0) and factor it for chunk length L, on stream s (NULL: the plan's).
 swr_status factor_for(swr_plan_t p, FactorSet& fs, int L, const double* V, double2* dg,
-                      double2* od, cudaStream_t s = nullptr) {
+                      double2* od, cudaStream_t s) {
     if (!s) s = p->s;
     if (fs.L != L || fs.nsteps != 1) {
         if (swr_factor_alloc(fs, p->N, L, chunks_for(p->nmax, L), s) != 0) return SWR_ERR_NOMEM;
@@ -1040,6 +1071,19 @@ swr_status upload_systems(MarchSys** dst, const std::vector<MarchSys>& v,
     if (st) return st;
     CK(cudaMemcpy(*dst, v.data(), sizeof(MarchSys) * v.size(), cudaMemcpyHostToDevice));
     if (p) p->host_sys.push_back({*dst, v});
+    return SWR_OK;
+}
+
+// Factors of their own for R g's lists (the build marches in FP64, at other chunk lengths).
+swr_status own_R(swr_plan_t p) {
+    const int L = p->fx_R.sh.L;
+    if (swr_factor_alloc(p->fsR, p->N, L, chunks_for(p->nmax, L), p->s) != 0) return SWR_ERR_NOMEM;
+    swr_status st = dalloc(&p->d_dgR, (size_t)p->ntot);
+    if (!st) st = dalloc(&p->d_odR, (size_t)p->ntot);
+    if (st) return st;
+    CK(cudaStreamCreateWithFlags(&p->fac_side, cudaStreamNonBlocking));
+    CK(cudaEventCreateWithFlags(&p->fac_fork, cudaEventDisableTiming));
+    CK(cudaEventCreateWithFlags(&p->fac_join, cudaEventDisableTiming));
     return SWR_OK;
 }
 
@@ -1724,6 +1768,7 @@ swr_status swr_test_wait_hook(int64_t max_polls, int32_t withhold) {
 void swr_destroy(swr_plan_t p) {
     if (!p) return;
     cudaStreamSynchronize(p->s);
+    if (p->fac_side) cudaStreamSynchronize(p->fac_side);
     cudaFree(p->d_n); cudaFree(p->d_goff); cudaFree(p->d_loff); cudaFree(p->d_tc);
     cudaFree(p->d_dg); cudaFree(p->d_od); cudaFree(p->d_dg0); cudaFree(p->d_od0);
     for (int k = 0; k < 5; ++k) {
@@ -1754,6 +1799,8 @@ void swr_destroy(swr_plan_t p) {
     for (auto& st : p->fx_side) cudaStreamDestroy(st);
     for (auto& e : p->fx_join) cudaEventDestroy(e);
     if (p->fx_fork) cudaEventDestroy(p->fx_fork);
+    swr_factor_free(p->fsR);
+    cudaFree(p->d_dgR); cudaFree(p->d_odR);
     if (p->fac_side) cudaStreamDestroy(p->fac_side);
     if (p->fac_fork) cudaEventDestroy(p->fac_fork);
     if (p->fac_join) cudaEventDestroy(p->fac_join);
@@ -2190,11 +2237,7 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
     if (!st && fx_one) {
         auto vr = apply_systems(p, 0), vf = apply_systems(p, SYS_WRITE_UT | SYS_TRACE);
         st = fx_list(p, p->fx_R, p->d_sys_R, vr.data(), p->N, 1, fx1, true);
-        if (!st && d->vkind == SWR_V_STATIC && !(fx && fxR == 3) &&
-            (cudaStreamCreateWithFlags(&p->fac_side, cudaStreamNonBlocking) != cudaSuccess ||
-             cudaEventCreateWithFlags(&p->fac_fork, cudaEventDisableTiming) != cudaSuccess ||
-             cudaEventCreateWithFlags(&p->fac_join, cudaEventDisableTiming) != cudaSuccess))
-            st = SWR_ERR_CUDA;
+        if (!st && d->vkind == SWR_V_STATIC && !(fx && fxR == 3)) st = own_R(p);
         if (!st && d->vkind == SWR_V_TIME) {
             auto vl = apply_systems(p, SYS_ZERO_U0);
             st = upload_systems(&p->d_sys_L, vl, p);
@@ -2271,27 +2314,16 @@ static swr_status build_body(swr_plan_t p, bool do_assemble) {
         // factorisations for the chunk lengths the marches of this plan will use
         const bool fx = p->fx_build.sys != nullptr;
         const int Lb = fx ? p->fx_build.sh.L : march_config(p, p->nsys_build).L;
-        const int La = p->fx_R.sys ? p->fx_R.sh.L : march_config(p, p->N).L;
+        const int La = p->fx_R.sys ? Lb : march_config(p, p->N).L;
         if ((st = factor_for(p, p->fsL[lidx(Lb)], Lb, p->d_V, p->d_dg, p->d_od))) return st;
         if (fx) LK(swr_launch_fx_prepare(p->fsL[lidx(Lb)], p->N, s, 0, 1, p->fx_hist));
-        // the factors of R g, where the build marches in FP64, beside those marches (22190 nodes in
-        // 3 subdomains, 79 steps: a build of 2.05 ms with them, 2.05 without, 2.13 in one stream)
-        const bool own = p->fx_R.sys && !fx, side = own && p->fac_side;
-        cudaStream_t sr = side ? p->fac_side : s;
-        if (side) {
-            CK(cudaEventRecord(p->fac_fork, s));
-            CK(cudaStreamWaitEvent(sr, p->fac_fork, 0));
-        }
-        if (La != Lb && (st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od, sr)))
+        if (La != Lb && (st = factor_for(p, p->fsL[lidx(La)], La, p->d_V, p->d_dg, p->d_od)))
             return st;
-        if (own) LK(swr_launch_fx_prepare(p->fsL[lidx(La)], p->N, sr, 0, 1, p->fx_hist));
-        if (side) CK(cudaEventRecord(p->fac_join, sr));
         CK(cudaMemsetAsync(p->d_iface, 0, sizeof(double2) * (nb + (size_t)p->ncols), s));
         // Algorithm 3, step 1: d and the first columns, 3 marches per interior subdomain
         st = run_march(p, false, p->d_sys_build, p->nsys_build, nullptr, p->d_iface, nullptr,
                        nullptr, p->d_u0, p->work_build);
         if (st) return st;
-        if (side) CK(cudaStreamWaitEvent(s, p->fac_join, 0));
         const double2* cols = p->d_iface + nb;
         LK(p_lag0(p, cols, p->d_lag0));
         if (p->d_hspec) LK(swr_launch_hist_spectra(p->N, p->nt, cols, p->d_hspec, s));
@@ -2406,6 +2438,9 @@ static swr_status fx_settle(swr_plan_t p, bool* changed) {
             continue;
         }
         c.fl->ran = false;
+        if (!c.zero && p->fx_R.sys && !p->fac_side) {   // R g had the build's factors
+            if ((st = own_R(p))) return st;
+        }
         if (!c.zero && p->superpose) {   // the FP64 marches' records: local node order
             p->rec_n = p->n;
             record_layout(p, p->rec_base);
@@ -2428,10 +2463,16 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
     cudaStream_t s = p->s;
     const size_t nb = (size_t)p->nb;
     const size_t nV = (p->d.vkind == SWR_V_TIME) ? (size_t)(p->nt + 1) * p->nx : p->nx;
+    if (p->uses_R) CK(cudaStreamWaitEvent(s, p->fac_join, 0));   // the last build's, which read d_V
+    p->have_R = false;
     CK(cudaEventRecord(p->ev[0], s));
     CK(cudaMemsetAsync(p->d_status, 0, sizeof(int), s));
     CK(cudaMemcpyAsync(p->d_V, V, sizeof(double) * nV, cudaMemcpyDeviceToDevice, s));
     CK(cudaMemcpyAsync(p->d_u0, u0, sizeof(double2) * p->nx, cudaMemcpyDeviceToDevice, s));
+    if (p->uses_R) {
+        CK(cudaEventRecord(p->fac_fork, s));
+        CK(cudaStreamWaitEvent(p->fac_side, p->fac_fork, 0));
+    }
     swr_status st = SWR_OK;
     if (p->tune.graph < 0) p->use_graph = false;
     const bool direct = !p->built || !p->use_graph;
@@ -2495,7 +2536,7 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
     if (p->d.vkind == SWR_V_STATIC) {       // the chunk lengths this build factors
         for (auto& f : p->fac_stale) f = true;
         p->fac_stale[lidx(p->fx_build.sys ? p->fx_build.sh.L : march_config(p, p->nsys_build).L)] = false;
-        p->fac_stale[lidx(p->fx_R.sys ? p->fx_R.sh.L : march_config(p, p->N).L)] = false;
+        if (!p->fx_R.sys) p->fac_stale[lidx(march_config(p, p->N).L)] = false;
     }
     if (!p->built || !p->use_graph) {
         st = build_body(p, false);
@@ -2544,6 +2585,10 @@ swr_status swr_build_interface(swr_plan_t p, const double* V, const double* u0) 
             p->gcount = 0;
             if ((st = build_body(p, true))) return st;
         }
+    }
+    if (p->uses_R) {
+        if ((st = form_R(p, p->fac_side))) return st;
+        CK(cudaEventRecord(p->fac_join, p->fac_side));
     }
     CK(cudaEventRecord(p->ev[1], s));
     st = read_status(p);
