@@ -35,34 +35,51 @@ FLOPS_PER_POINT_STEP_TDEP = 56     # plus the per-step factorisation (one comple
 # factors (36) plus the generalised-mass term b_f(zeta) (30) and the convergence test (10)
 FLOPS_PER_POINT_ITER_NL = 76
 FP64_PEAK_GFLOPS = 152 * 2 * 2 * 2.07   # SMs x FP64 FMA/clk x 2 flop x GHz (max SM clock)
-# The linear marches run in 64-bit fixed point (k_march_fx): per warp and node-step five complex
-# multiply-adds of 12 mad.wide.s32 (2.13 cycles each, measured) and about 100 cycles of
-# additions, shifts and rounding, 230 in all, on 608 SM sub-partitions.  Their roof is that
-# issue rate, in the same algorithmic flops per node-step.
-FX_CYCLES = 230
+# The linear marches run in 64-bit fixed point where a plan's counts say so (k_march_fx).  Their
+# roof is the issue rate of the multiply-adds alone: per warp and node-step five complex ones of
+# 12 mad.wide.s32, 2.13 cycles each (measured), on 608 SM sub-partitions, in the same
+# algorithmic flops per node-step.
+FX_CYCLES = 5 * 12 * 2.13
 FX_PEAK_GFLOPS = 608 * 2.07 * 32 / FX_CYCLES * FLOPS_PER_POINT_STEP
-FX_BASIS = ("issue rate of the 64-bit fixed-point march (%d cycles per warp and node-step on 608 SM "
-            "sub-partitions at 2070 MHz) in FP64-equivalent flops" % FX_CYCLES)
+FX_BASIS = ("issue rate of the fixed-point march's integer multiply-adds (60 of 2.13 cycles per warp and "
+            "node-step on 608 SM sub-partitions at 2070 MHz) in FP64-equivalent flops")
 
-# DRAM bytes (read + write) per march launch, each scaled by the steps from 100-step
-# single-launch ncu captures (profiles/k_march_static_N500_build.md, launch_list_scaling.md,
-# launch_list_timedep.md).  Scaling step: the mean over its four build marches, the N = 500
-# build (lean k_march_static<12>: 19.1 MB read, 593.5 MB written per 100 steps, the recorded
-# states) standing for N = 256 and the N = 16 build (k_march_tl<12>: 19.2 / 547.0 MB) for
-# N = 64.  V(t,x) march: the streamed per-step factors, 677.2 MB read and 0.3 MB written per
-# 100 steps (captured on k_march_static's general instantiation in the modelled cluster
-# shape, whose code the later k_march_tl changes did not touch; the lean one of the tuned
-# shape streams the same factors, 7.1 MB per step in its 38-step probes).  Valid only for
-# the march sources they were taken from (sha256 prefix of swr_march.cu +
-# swr_internal.cuh), null otherwise.
-MARCH_TRAFFIC = {"sources": "647131b39d98daf0",
-                 "scaling": 2947000000.0, "timedep": 6775000000.0}
+# DRAM bytes (read + write) per march launch, each scaled by the steps from 100-step (16
+# subdomains: 200-step) single-launch ncu captures (profiles/k_march_fx_forms.md).  Scaling step:
+# the mean over its four build marches (16, 64, 256 and 500 subdomains: 5.86, 6.05, 6.30 and
+# 6.35 MB a step, nearly all of it the recorded states written once).  V(t,x) march: the
+# per-step rows of coefficients, 5.99 MB a step.  Valid only for the march sources they were
+# taken from (sha256 prefix), null otherwise.
+MARCH_SOURCES = ("swr_march_fx.cu", "swr_fx.cuh", "swr_internal.cuh")
+MARCH_TRAFFIC = {"sources": "f60d8a1e80bb58b3",
+                 "scaling": 3071000000.0, "timedep": 5994000000.0}
+
+
+def march_form(plans):
+    """What the plans' main marches (the build's, or R's for V(t,x)) last ran as: the kernel's name
+    and (systems in fixed point, of them marched again in FP64, plans wholly in FP64)."""
+    n = again = f64 = 0
+    for p in plans:
+        c = p.fixed_point_counts()
+        k = max((c["build"], c["R"], c["L"]), key=lambda v: v[0])
+        n, again, f64 = n + k[0], again + k[1], f64 + (k[0] == 0)
+    name = "k_march_static" if n == 0 else "k_march_fx"
+    if n and (again or f64):
+        name = "k_march_fx (%d of %d systems again in FP64, %d of %d plans in FP64)" % (
+            again, n, f64, len(plans))
+    return name, (n, again, f64)
+
+
+def march_roof(plans, peak):
+    """The kernel the plans' marches ran, its roof and what that is (peak: the FP64 one)."""
+    name, (n, again, f64) = march_form(plans)
+    return (name, FX_PEAK_GFLOPS, FX_BASIS) if n else (name, peak[0], peak[1])
 
 
 def march_sources_hash():
     import hashlib
     h = hashlib.sha256()
-    for f in ("swr_march.cu", "swr_internal.cuh"):
+    for f in MARCH_SOURCES:
         with open(os.path.join(ROOT, "paper_1503_02564_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -508,6 +525,7 @@ def run_batch(args, peak=None):
     launches = swr.swr_kernel_launch_count() - launches0
     clocks = sampler.stop()
     st = plan.get_stats(reset=True)
+    m_kernel, roof, basis = march_roof([plan], peak)
     t_s, its = timed(one_by_one)
     u_b = uT.cpu().numpy()
     k, dev_max = 0, 0.0
@@ -565,13 +583,13 @@ def run_batch(args, peak=None):
                    "subdomains": int(sum(w.nsub for w in wls)),
                    "point_steps_per_step": ps, "l2": "flushed by a 256 MB write before each step",
                    "parallelism": "single GPU"},
-        "roofline": {"kernel": "k_march_fx", "bound": "alu", "achieved": achieved,
-                     "peak": FX_PEAK_GFLOPS, "unit": "GFLOP/s",
-                     "frac": achieved / FX_PEAK_GFLOPS, "traffic": None,
+        "roofline": {"kernel": m_kernel, "bound": "alu", "achieved": achieved,
+                     "peak": roof, "unit": "GFLOP/s",
+                     "frac": achieved / roof, "traffic": None,
                      "launches": st["march_launches"],
                      "avg_launch_ms": st["march_ms"] / max(st["march_launches"], 1),
                      "flops_per_point_step": FLOPS_PER_POINT_STEP,
-                     "peak_basis": FX_BASIS, "ratio_to_fp64_rate": achieved / peak[0]},
+                     "peak_basis": basis, "ratio_to_fp64_rate": achieved / peak[0]},
         "per_instance_plans": {"ms_per_step": t_s / args.steps,
                                "speedup_of_batched": t_s / t_b,
                                "iterations_min_max": [min(its), max(its)],
@@ -749,6 +767,7 @@ def run_plain(args, dev, local, peak):
     achieved = FLOPS_PER_POINT_STEP * st["march_point_steps"] / (st["march_ms"] * 1e-3) / 1e9
     hV, hu0 = V.cpu().pin_memory(), u0.cpu().pin_memory()
     huT = torch.empty(wl.nx, dtype=torch.complex128).pin_memory()
+    m_kernel, roof, basis = march_roof([plan], peak)
     e_ms, _, _ = timed(plan, (hV, hu0, huT))
     plan.destroy()
     cpu = None
@@ -776,9 +795,9 @@ def run_plain(args, dev, local, peak):
                                "(GMRES(30), causal preconditioner) vs classical, to 1e-10",
                    "l2": "flushed by a 256 MB write before each solve"},
         "algorithms": rows,
-        "roofline": {"kernel": "k_march_fx", "bound": "alu", "achieved": achieved,
-                     "peak": FX_PEAK_GFLOPS, "unit": "GFLOP/s", "frac": achieved / FX_PEAK_GFLOPS,
-                     "traffic": None, "peak_basis": FX_BASIS,
+        "roofline": {"kernel": m_kernel, "bound": "alu", "achieved": achieved,
+                     "peak": roof, "unit": "GFLOP/s", "frac": achieved / roof,
+                     "traffic": None, "peak_basis": basis,
                      "ratio_to_fp64_rate": achieved / peak[0],
                      "flops_per_point_step": FLOPS_PER_POINT_STEP,
                      "note": "4 systems of 251 nodes: latency-bound, one CTA per system"},
@@ -1038,14 +1057,16 @@ def run_workload(args, workload, rank, world, local, dev, peak):
     variant = st[0]["march_variant"]
     traffic = None
     if (march_sources_hash() == MARCH_TRAFFIC["sources"] and args.nt == 0 and args.tc == "robin"
-            and (timedep or tuple(nsubs) == NSUBS)):
+            and not adjoint and (timedep or tuple(nsubs) == NSUBS)
+            and march_form([c["plan"] for c in cases])[0] == "k_march_fx"):
         traffic = MARCH_TRAFFIC["timedep" if timedep else "scaling"]
     streamed = variant == swr.MARCH_TDEP_STREAMED
     fpp = FLOPS_PER_POINT_STEP_TDEP if variant == swr.MARCH_TDEP_REFACTOR else FLOPS_PER_POINT_STEP
-    fixed = not (variant == swr.MARCH_TDEP_REFACTOR or adjoint or nonlin
-                 or (tuning_of(args) or {}).get("two_level", 0) < 0)
+    # (the adjoint's time is in its segment marches, FP64)
+    form = march_form([c["plan"] for c in cases])
+    fixed = form[1][0] > 0 and not adjoint
     m_kernel = ("k_march_tdep" if variant == swr.MARCH_TDEP_REFACTOR else
-                "k_march_fx" if fixed else "k_march_static")
+                "k_march_static" if adjoint else form[0])
     dfma_gf = peak_gf
     if fixed:
         peak_gf, peak_basis = FX_PEAK_GFLOPS, FX_BASIS
@@ -1152,6 +1173,8 @@ def run_workload(args, workload, rank, world, local, dev, peak):
                           "causal_window": st[len(per_n)]["causal_window"],
                           "superposed": st[len(per_n)]["superposed"],
                           "toeplitz_fft_length": st[len(per_n)]["toeplitz_fft_length"],
+                          "fixed_point": {k: v for k, v in c["plan"].fixed_point_counts().items()
+                                          if v[0]},
                           "residual": info["residual"], "build_ms": info["t_build_ms"],
                           "solve_ms": info["t_solve_ms"], "final_ms": info["t_final_ms"],
                           "interface_jump": info["interface_jump"]})

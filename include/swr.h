@@ -158,7 +158,8 @@ typedef struct swr_tuning {
                                 /* a system has <= 993 separators (the nonlinear         */
                                 /* gradient's monodomain: <= 8161); -1 cluster-wide PCR, */
                                 /* and the linear marches in FP64 instead of 64-bit      */
-                                /* fixed point (Robin, Neumann and S_0^2 ends, nt >= 16) */
+                                /* fixed point (Robin, Neumann and, for dt >= 32 h^2,    */
+                                /* S_0^2 ends, nt >= 16; see swr_fixed_point_counts)     */
     int32_t debug;              /* 1: failing CUDA calls (2: also the launch-shape      */
                                 /* probes) reported on stderr; 0 (default) silent        */
     int32_t history_fft;        /* causal substitution (CAUSAL preconditioner, direct   */

@@ -16,7 +16,8 @@
 // limbs give the dropped term no mean: with an unsigned Xl it is a constant of up to one
 // unit per coefficient, the same at every step, and 200 steps of the plain workload then
 // ended 1.3e-13 off instead of 4e-14 in FP64.  Splitting at 32 bits costs one or two
-// instructions (the low limb is the low register).
+// instructions (the low limb is the low register).  Where even two units show (coarse grids,
+// S_0^2 ends: fx_full in swr_capi.cu) the last term is taken too (fx_mac_full).
 //
 // No accumulator wraps: over the (at most six) real products of one component, two of them
 // with |X| < 2^61 and the others with |X| < 2^60,

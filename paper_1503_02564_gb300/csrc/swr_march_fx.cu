@@ -38,11 +38,13 @@
 // see k_fx_flux) are marched again in FP64 by the kernels of swr_march.cu.  The first step,
 // which sets the scale, is always an FP64 one.
 //
-// Measured, build marches of 200001 nodes and 500 steps (zero flux, left and right impulse),
-// FP64 -> here: 500 subdomains 16.9 -> 4.5 ms, 256 19.4 -> 5.9, 64 19.3 -> 5.9, 16 20.1 -> 9.2
-// (bound by issue, about 240 instructions per node and step at 500; by a step's dependent
-// chain and its separators' exchange at 16).  V(t,x), 60001 nodes in 64 subdomains, 400 steps:
-// 4.7 -> 2.2 ms a march (one CTA of six warps per subdomain: the chain of a step, 5.6 us).
+// Measured, build marches of 200001 nodes and 500 steps (zero flux, left and right impulse; first
+// step, scales, march and fluxes), FP64 -> here: 500 subdomains 16.6 -> 4.7 ms, 256 19.4 -> 6.3, 64
+// 18.9 -> 6.3, 16 19.5 -> 10.3 (bound by issue, about 240 instructions per node and step at 500; by
+// a step's dependent chain and its separators' exchange at 16).  S_0^2 ends, 100003 nodes in 61
+// subdomains, 300 steps: 7.5 -> 4.1.  1001 nodes in 4 subdomains, 200 steps, whole products: 1.65
+// -> 1.01.  V(t,x), 60001 nodes in 64 subdomains, 400 steps: 4.76 -> 2.26 ms a march (one CTA of
+// six warps per subdomain: the chain of a step, 5.6 us).
 #include <cooperative_groups.h>
 
 #include <algorithm>
@@ -1048,9 +1050,11 @@ bool swr_fx_shape(int nmax, int ngroups, int R, int forceL, int nsm, FxShape* ou
             const double warps = ctas * R * (T / 32) / 4.0;   // per SM sub-partition
             double step = waves * std::max(lat, std::max(warps, 1.0) * iss);
             // four-node chunks only where they are clearly faster: the factors of more separators
-            // carry more rounding error (R g of 200001 nodes, 256 subdomains, 500 steps, against
-            // extended precision: 5.8e-12 with 4 nodes, 3.3e-12 with 8, 2.7e-12 with 12, in FP64
-            // the same) and the march gains nothing (that R g: 3.65 ms with 4, 3.54 ms with 8)
+            // carry more rounding error, the same here and in FP64 (the build's columns of 20 drawn
+            // problems of 5000 to 85000 nodes against extended precision: larger than with eight
+            // nodes in 17, by 9 % in the mean; d and R g alike).  On 15 problems the factor chose
+            // eight nodes twice where four were faster (14019 nodes in 28 subdomains, 150 steps: 1.29
+            // against 1.09 ms a build; 76618 in 138: 1.32, 1.26).
             if (L == 4 && !stream) step *= 1.25;
             if (best < 0.0 || step < best) {
                 best = step;
