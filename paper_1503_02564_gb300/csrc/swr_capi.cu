@@ -178,7 +178,8 @@ struct swr_plan_s {
     std::vector<cudaStream_t> fx_side;   // launches of a list beside the first
     cudaEvent_t fx_fork = nullptr;
     std::vector<cudaEvent_t> fx_join;
-    // R g in fixed point, the build in FP64: R g's factors and matrix (see form_R)
+    // R g in fixed point, the build in FP64 or at another chunk length: R g's factors and matrix
+    // (see form_R)
     FactorSet fsR;
     double2 *d_dgR = nullptr, *d_odR = nullptr;
     bool uses_R = false, have_R = false;
@@ -1074,7 +1075,7 @@ swr_status upload_systems(MarchSys** dst, const std::vector<MarchSys>& v,
     return SWR_OK;
 }
 
-// Factors of their own for R g's lists (the build marches in FP64, at other chunk lengths).
+// Factors of their own for R g's lists (the build marches in FP64, or at another chunk length).
 swr_status own_R(swr_plan_t p) {
     const int L = p->fx_R.sh.L;
     if (swr_factor_alloc(p->fsR, p->N, L, chunks_for(p->nmax, L), p->s) != 0) return SWR_ERR_NOMEM;
@@ -2093,17 +2094,16 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
     const bool fx = fxR > 0 && fx_tc && !is_long && p->two_level && crossed &&
                     p->nt >= 16 &&
                     swr_fx_shape(p->nmax, p->N, fxR, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fxs);
-    // the marches of one system per subdomain (R g, final, the adjoint's d), with the build's
-    // chunk length where that has a fixed-point form: one set of factors, formed by the build.  (A
-    // length of their own, factored by the build as well, moved R g by -16 to +28 % on ten problems
-    // of 5000 to 160000 nodes and the build by 0 to 13 %; 256 subdomains of 782 nodes, 500 steps:
-    // R g 3.52 instead of 3.77 ms, the build 6.94 instead of 6.74.)
+    // the marches of one system per subdomain (R g, final, the adjoint's d): a chunk length of their
+    // own, with factors of their own where it is not the build's (see form_R).  (With the build's,
+    // R g took from 16 % less to 28 % more on ten problems of 5000 to 160000 nodes; 256
+    // subdomains of 782 nodes, 500 steps: 3.77 ms instead of 3.52.)
     FxShape fx1{};
     const bool fx_one = d->vkind != SWR_V_NONLINEAR && fx_tc && !is_long &&
                         p->two_level && p->nt >= 16 &&
                         (d->vkind != SWR_V_TIME || p->tune.tdep_precomp >= 0) &&
-                        swr_fx_shape(p->nmax, p->N, 1, fx && fxR == 3 ? fxs.L : (p->forceL == 2 ? 0 : p->forceL),
-                                     p->nsm, &fx1, d->vkind == SWR_V_TIME);
+                        swr_fx_shape(p->nmax, p->N, 1, p->forceL == 2 ? 0 : p->forceL, p->nsm, &fx1,
+                                     d->vkind == SWR_V_TIME);
     p->rec_n.resize(p->N);
     for (int j = 0; j < p->N; ++j)   // chunk-element order: (L + 1) rows of P_j + 1
         p->rec_n[j] = fx && fxR == 3 ? (fxs.L + 1) * (chunks_for(p->n[j], fxs.L) + 1) : p->n[j];
@@ -2237,7 +2237,7 @@ static swr_status plan_create(const swr_desc* ds, int count, const swr_tuning* t
     if (!st && fx_one) {
         auto vr = apply_systems(p, 0), vf = apply_systems(p, SYS_WRITE_UT | SYS_TRACE);
         st = fx_list(p, p->fx_R, p->d_sys_R, vr.data(), p->N, 1, fx1, true);
-        if (!st && d->vkind == SWR_V_STATIC && !(fx && fxR == 3)) st = own_R(p);
+        if (!st && d->vkind == SWR_V_STATIC && !(fx && fxR == 3 && fx1.L == fxs.L)) st = own_R(p);
         if (!st && d->vkind == SWR_V_TIME) {
             auto vl = apply_systems(p, SYS_ZERO_U0);
             st = upload_systems(&p->d_sys_L, vl, p);

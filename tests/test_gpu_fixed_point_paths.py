@@ -228,10 +228,9 @@ def test_first_march_after_a_build_is_like_the_next(nx, nsub, tc):
         n0 = swr.swr_kernel_launch_count()
         out.append(apply_R(plan, g))
         launches.append(swr.swr_kernel_launch_count() - n0)
-    in_build = plan.fixed_point_counts()["build"][0] > 0
     plan.destroy()
-    # (where the build marches in FP64, the plan's very first march of R g forms its factors)
-    assert launches[1] == launches[2] == launches[3] and (launches[0] == launches[1] or not in_build)
+    # (where R g has a chunk length of its own, the plan's very first march of it forms the factors)
+    assert launches[0] >= launches[1] == launches[2] == launches[3]
     assert np.array_equal(out[1], out[2]) and np.array_equal(out[2], out[3])
     wl.V = wl.V * 2.0
     assert rel(out[1], O.apply_R(problem(wl, tc), g)) < TOL_MARCH
