@@ -51,7 +51,7 @@ FX_BASIS = ("issue rate of the fixed-point march's integer multiply-adds (60 of 
 # per-step rows of coefficients, 5.99 MB a step.  Valid only for the march sources they were
 # taken from (sha256 prefix), null otherwise.
 MARCH_SOURCES = ("swr_march_fx.cu", "swr_fx.cuh", "swr_internal.cuh")
-MARCH_TRAFFIC = {"sources": "f60d8a1e80bb58b3",
+MARCH_TRAFFIC = {"sources": "7e9339e393d0875c",
                  "scaling": 3071000000.0, "timedep": 5994000000.0}
 
 

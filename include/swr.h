@@ -449,6 +449,9 @@ swr_status swr_fp64_peak(int32_t kind, int64_t iters, int32_t blocks, int32_t th
  *   max_polls: the poll limit of those waits (<= 0: the default);
  *   withhold:  an interface (global index) whose CTA never publishes its progress,
  *              so that its neighbours' waits run out (< 0: none, the default).
+ * The fixed-point marches (swr_fixed_point_counts) take both too: their waits are for the
+ * rows of a subdomain spread over a cluster and, V(t,x), for a step's factors, and the
+ * subdomain of that index hands on neither.
  * Affects launches enqueued after the call; restore with (0, -1).
  * Errors: SWR_ERR_CUDA. */
 swr_status swr_test_wait_hook(int64_t max_polls, int32_t withhold);

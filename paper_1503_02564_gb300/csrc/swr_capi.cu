@@ -1763,6 +1763,7 @@ const char* swr_status_string(swr_status s) {
 int64_t swr_kernel_launch_count(void) { return (int64_t)g_launches.load(); }
 
 swr_status swr_test_wait_hook(int64_t max_polls, int32_t withhold) {
+    swr_fx_set_wait_hook((long long)max_polls, (int)withhold);
     return swr_set_wait_hook((long long)max_polls, (int)withhold) == 0 ? SWR_OK : SWR_ERR_CUDA;
 }
 

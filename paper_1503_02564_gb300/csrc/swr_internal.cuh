@@ -302,6 +302,7 @@ struct FxMarchArgs {
     const double2* u0;
     double2* htrace;
     double2 two_c2;
+    int polls, withhold;  // limit of a wait; test hook: the subdomain that hands nothing on (-1: none)
     int full;             // all products whole (coarse grids; S_0^2 ends always)
     // per-step factors: subdomains N, the step-1 set and the direction of the walk
     int stream, N, fstep0, frev;
@@ -381,6 +382,7 @@ int swr_fx_alloc_steps(FactorSet& fs, int N);
 int swr_launch_fx_start(const FactorSet& fs, FxMarchArgs a, int nsys, const double2* gin,
                         double2 inv_ik, cudaStream_t s);
 int swr_launch_march_fx(const FactorSet& fs, FxMarchArgs a, int ngroups, cudaStream_t s);
+void swr_fx_set_wait_hook(long long polls, int withhold);
 int swr_launch_fx_flux(const FxMarchArgs& a, int nsys, double2 two_sigma, const double2* gin,
                        double2* gout, double2* vtrace, cudaStream_t s);
 int swr_launch_superpose_fx(const FactorSet& fs, const double2* urec, const long long* rec_base,

@@ -48,6 +48,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <atomic>
 
 #include "swr_fx.cuh"
 #include "swr_internal.cuh"
@@ -458,9 +459,10 @@ __device__ __forceinline__ void fx_push(unsigned addr, unsigned mbar, FxC x) {
     asm volatile("st.async.weak.shared::cluster.mbarrier::complete_tx::bytes.v2.b64 [%0], {%1, %2}, [%3];"
                  ::"r"(addr), "l"(x.r), "l"(x.i), "r"(mbar) : "memory");
 }
-// wait for the phase of this parity; false after about a second (the caller flags a timeout)
-__device__ __forceinline__ bool fx_wait(unsigned mbar, unsigned parity) {
-    for (int k = 0; k < 1000000; ++k) {
+// wait for the phase of this parity; false after `polls` polls of up to a microsecond (a million:
+// about a second; the caller flags a timeout)
+__device__ __forceinline__ bool fx_wait(unsigned mbar, unsigned parity, int polls) {
+    for (int k = 0; k < polls; ++k) {
         unsigned ok;
         asm volatile("{\n\t.reg .pred q;\n\t"
                      "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 q, [%1], %2, 1000;\n\t"
@@ -542,6 +544,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
     // rows of the separators this CTA holds (one contiguous piece), zero beyond them.  STREAM:
     // step t's rows and reduced system go to buffer t & 1 by one bulk copy each
     auto fetch = [&](int t) {
+        if (j == a.withhold) return;   // false but under the test hook
         const size_t st = a.fstep0 + (a.frev ? 1 - t : t - 1);
         const unsigned dst = fx_saddr(fsm + (t & 1) * BUF), mb = fx_saddr(full + (t & 1));
         asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mb),
@@ -640,7 +643,8 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
     bool grown = false, late = false;
     int tlate = 0;   // STREAM: the step whose wait ran out
     const int nw = Pj / 32 + 1;            // warps of the system that hold separators
-    const int ncta = Pj / T + 1;           // CTAs of the cluster that do
+    // CTAs of the cluster that do (none to push to under the test hook)
+    const int ncta = j == a.withhold ? 0 : Pj / T + 1;
     // bytes a step pushes to each of them: A[0..Q], and B of every warp whose lane 31 is not
     // the system's last separator
     const unsigned txb = 16u * (Q + 1 + nw - ((Pj & 31) == 31 ? 1 : 0));
@@ -675,7 +679,7 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                 __syncwarp();   // the other buffer has been read
                 if (tid == 0 && t < nsteps) fetch(t + 1);
             }
-            late = !fx_wait(fx_saddr(full + (t & 1)), ((t - 2) >> 1) & 1);
+            late = !fx_wait(fx_saddr(full + (t & 1)), ((t - 2) >> 1) & 1, a.polls);
             late = __any_sync(0xffffffffu, late);
             // a system of several warps in one CTA gives up together, at the step's barrier
             if (late && (ONE || C > 1 || T == 32)) {
@@ -825,10 +829,10 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
                 }
             }
             if (C > 1) {
-                late = !fx_wait(fx_saddr(mbar + par * R + r), ((t - 2) >> 1) & 1);
+                late = !fx_wait(fx_saddr(mbar + par * R + r), ((t - 2) >> 1) & 1, a.polls);
                 if (__any_sync(0xffffffffu, late)) {   // give up; a last bounded wait for rows in flight
                     late = true;
-                    fx_wait(fx_saddr(mbar + par * R + r), ((t - 2) >> 1) & 1);
+                    fx_wait(fx_saddr(mbar + par * R + r), ((t - 2) >> 1) & 1, a.polls);
                     break;
                 }
             } else if (STREAM && T > 32) {
@@ -935,8 +939,9 @@ __global__ void __launch_bounds__(L == 16 ? 256 : (L == 4 && !STREAM ? 512 : 384
     if (valid && ((mu >> 27) || (mv >> 27) || late)) a.bad[sidx] = 1;
     if (late) atomicOr(a.status, ST_TIMEOUT);
     if (STREAM && tlate && tid == 0) {   // copies in flight, once more within the limit
-        fx_wait(fx_saddr(full + (tlate & 1)), ((tlate - 2) >> 1) & 1);
-        if (ONE && tlate < nsteps) fx_wait(fx_saddr(full + ((tlate + 1) & 1)), ((tlate - 1) >> 1) & 1);
+        fx_wait(fx_saddr(full + (tlate & 1)), ((tlate - 2) >> 1) & 1, a.polls);
+        if (ONE && tlate < nsteps)
+            fx_wait(fx_saddr(full + ((tlate + 1) & 1)), ((tlate - 1) >> 1) & 1, a.polls);
     }
     if (valid && (sy.flags & (SYS_REC_LAST | SYS_WRITE_UT))) {
         const double s1 = fx_pow2(sh - sc);
@@ -1126,7 +1131,17 @@ int swr_launch_fx_start(const FactorSet& fs, FxMarchArgs a, int nsys, const doub
     return cudaGetLastError() == cudaSuccess ? 0 : -1;
 }
 
+// Test hook of the waits (swr_test_wait_hook): taken by the launches enqueued after it.
+static std::atomic<long long> g_fx_polls{1000000};
+static std::atomic<int> g_fx_withhold{-1};
+void swr_fx_set_wait_hook(long long polls, int withhold) {
+    g_fx_polls = polls > 0 ? std::min(polls, 1000000LL) : 1000000LL;
+    g_fx_withhold = withhold;
+}
+
 int swr_launch_march_fx(const FactorSet& fs, FxMarchArgs a, int ngroups, cudaStream_t s) {
+    a.polls = (int)g_fx_polls;
+    a.withhold = g_fx_withhold;
     a.P = fs.P;
     a.sub_P = fs.sub_P;
     a.sep_pos = fs.sep_pos;
